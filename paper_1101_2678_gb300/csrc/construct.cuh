@@ -43,6 +43,10 @@ struct GroupSmem {
   long long wlen[4];
   int wmin[4];
   int next;
+  // the walk with compaction
+  float wtot[4];
+  int fnext[2], chosen, slot;
+  int xnext, xchosen, xslot;
 };
 
 constexpr int kMaxGroupsPerCta = 8;
@@ -269,6 +273,19 @@ struct Seg {
       const unsigned long long t = shfl_up(x, o);
       if (hl >= o) x += t;
     }
+    return x;
+  }
+  // Inclusive sums in single precision; the shuffle's own predicate says
+  // whether a lane d below exists in the segment.
+  __device__ __forceinline__ float inclusive_scan_f(float x) const {
+#pragma unroll
+    for (int o = 1; o < H; o <<= 1)
+      asm volatile(
+          "{\n\t.reg .pred p;\n\t.reg .f32 t;\n\t"
+          "shfl.sync.up.b32 t|p, %0, %1, %2, %3;\n\t"
+          "@p add.rn.f32 %0, %0, t;\n\t}"
+          : "+f"(x)
+          : "r"(o), "n"((32 - H) << 8), "r"(mask));
     return x;
   }
   __device__ __forceinline__ void sync() const { __syncwarp(mask); }

@@ -46,23 +46,151 @@ struct WalkState {
   int cur;       // current city
   int s;         // next step (1 .. n-1)
   int live;      // unvisited cities listed for the current phase (gather phases)
-  unsigned long long rwin;  // this lane's Philox words for the steps of the window
+  float u;       // this lane's uniform r / 2^64 for its step of the window
   uint32_t parity;          // mbarrier phase of the row copy
   bool waits_ok;
 };
+
+// The city of one step: `next`, and in gather phases the thread and slot that
+// hold it (chosen = -1: already marked).
+struct Pick {
+  int next, chosen, slot;
+};
+
+// The integer roulette of one step from the staged row (reading R2), slot by
+// slot: taken when the float search below cannot tell which city the target
+// falls on, or no open weight is positive.  A call of its own, so that it
+// costs the walk neither registers nor instructions (0.1-2 % of the steps).
+// list = nullptr: slot i of thread tg is city tg*cp + i with tabu bits v0..v2;
+// otherwise the list entry tg*cp + i.
+template <int G, int H, uint32_t kUnit>
+__device__ __noinline__ Pick exact_pick(const float* row, uint16_t* list, int cp, uint32_t zero_entry,
+                                        uint32_t v0, uint32_t v1, uint32_t v2, int tg, int bar_id,
+                                        GroupSmem* gs, unsigned long long r) {
+  constexpr int NT = G * H;
+  const Seg<H> seg(threadIdx.x & 31);
+  const int hl = seg.hl, wg = G > 1 ? tg >> 5 : 0;
+  auto group_wait = [&]() {
+    if constexpr (G > 1)
+      group_sync(bar_id, NT);
+    else
+      seg.sync();
+  };
+  auto weight = [&](int i) -> uint32_t {
+    if (list) return entry_weight<kUnit>(row, list[tg * cp + i]);
+    const uint32_t word = i < 32 ? v0 : (i < 64 ? v1 : v2);
+    return (word >> (i & 31)) & 1u ? 0u : __float_as_uint(row[tg * cp + i]);
+  };
+  uint32_t mx = 0u;
+#pragma unroll 4
+  for (int i = 0; i < cp; ++i) mx = max(mx, weight(i));
+  mx = seg.max_u32(mx);
+  if constexpr (G > 1) {
+    if (hl == 0) gs->wmax[wg] = mx;
+    group_wait();
+#pragma unroll
+    for (int k = 0; k < G; ++k) mx = max(mx, gs->wmax[k]);
+  }
+  if (mx == 0u) {
+    // Every open weight is zero: the lowest open city (a list's smallest
+    // entry; zero_entry is above every city's).
+    uint32_t cand = 0xffffffffu;
+    for (int i = cp - 1; i >= 0; --i) {
+      if (list) {
+        cand = min(cand, (uint32_t)list[tg * cp + i]);
+      } else {
+        const uint32_t word = i < 32 ? v0 : (i < 64 ? v1 : v2);
+        if (!((word >> (i & 31)) & 1u)) cand = (uint32_t)(tg * cp + i);
+      }
+    }
+    cand = seg.min_u32(cand);
+    if constexpr (G > 1) {
+      if (hl == 0) gs->wmin[wg] = (int)cand;
+      group_wait();
+#pragma unroll
+      for (int k = 0; k < G; ++k) cand = min(cand, (uint32_t)gs->wmin[k]);
+    }
+    if (!list) return Pick{(int)cand, -1, 0};
+    // no other thread reads these entries until the step's end
+    for (int i = 0; i < cp; ++i)
+      if (list[tg * cp + i] == cand) list[tg * cp + i] = (uint16_t)zero_entry;
+    return Pick{(int)(cand / kUnit), -1, 0};
+  }
+  float f1, f1s, f2;
+  quant_factors(kRouletteBits - 1 - exponent_of_bits(mx), f1, f1s, f2);
+  unsigned long long mine = 0;
+#pragma unroll 4
+  for (int i = 0; i < cp; ++i) mine += quant_value(weight(i), f1, f1s, f2);
+  const unsigned long long incl = seg.inclusive_scan(mine);
+  const unsigned long long wtot = seg.shfl(incl, H - 1);
+  unsigned long long woff = 0, Q = wtot;
+  if constexpr (G > 1) {
+    if (hl == 0) gs->wsum[wg] = wtot;
+    group_wait();
+    Q = 0;
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      const unsigned long long v = gs->wsum[k];
+      if (k < wg) woff += v;
+      Q += v;
+    }
+  }
+  const unsigned long long T = __umul64hi(r, Q);
+  Pick out{0, 0, 0};
+  if (G == 1 || (T >= woff && T - woff < wtot)) {
+    const int L = max(__ffs(seg.ballot(woff + incl > T)) - 1, 0);
+    int slot = 0, city = 0;
+    if (hl == L) {
+      unsigned long long c = woff + incl - mine;
+      for (; slot < cp - 1; ++slot) {
+        c += quant_value(weight(slot), f1, f1s, f2);
+        if (c > T) break;
+      }
+      city = list ? (int)(list[tg * cp + slot] / kUnit) : tg * cp + slot;
+    }
+    out.next = seg.shfl(city, L);
+    out.chosen = wg * 32 + L;
+    out.slot = seg.shfl(slot, L);
+    if constexpr (G > 1) {
+      if (hl == 0) {
+        gs->xnext = out.next;
+        gs->xchosen = out.chosen;
+        gs->xslot = out.slot;
+      }
+    }
+  }
+  if constexpr (G > 1) {
+    group_wait();
+    out = Pick{gs->xnext, gs->xchosen, gs->xslot};
+  }
+  return out;
+}
 
 // Steps [w.s, s_end) of one phase.  CP: slots per thread.  kGather = false:
 // slot i of thread t is city t*C + i (phase 0); true: slot i holds the entry
 // ulist[t*CP + i] (its city's weight, or the zero slot once visited).  CPN > 0:
 // afterwards, list the unvisited cities for a phase of CPN slots per thread.
+//
+// A step samples the integer roulette without its integers.  With S the sum
+// of the open weights and u = r / 2^64, the roulette takes the city whose
+// interval of the prefix sums holds u S, up to the floors of its quantiser:
+// at most n 2^-45 S.  The step forms the prefix sums in single precision
+// (per part of a thread's slots, a warp scan over the threads, a second scan
+// over the chosen part) and takes the city only if u S lies inside its
+// interval by more than eps S on both sides, eps = kRoundings 2^-24: every
+// partial sum of non-negative terms is within (its roundings) 2^-24 S of the
+// true one, so the integer roulette takes the same city.  Otherwise (the
+// target within the error of a boundary; S zero, tiny, infinite or NaN) the
+// step runs exact_pick().  This drops the max pass, the three FMAs of the
+// quantiser and half of every shuffle (64-bit scans) from a step.
 template <int C, int CP, int CPN, int G, int H, bool kGather, bool kPool>
 __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, const int tg,
                                           const Seg<H> seg, GroupSmem* gs, const int bar_id,
                                           float* srow, uint16_t* ulist, const int start,
                                           const int s_end, WalkState& w, const bool lane_copy) {
-  static_assert(CP % 4 == 0 && CP >= 4 && CP <= 128, "CP must be a multiple of 4 in [4,128]");
+  static_assert(CP % 4 == 0 && CP >= 4 && CP <= 96, "CP must be a multiple of 4 in [4,96]");
   static_assert(kGather || CP == C, "the direct phase reads whole chunks");
-  static_assert(G == 1 || (G == 2 && H == 32), "two warps per ant use whole warps");
+  static_assert(G == 1 || H == 32, "several warps per ant use whole warps");
   constexpr int NT = G * H;  // threads per ant
   constexpr int NW = (CP + 31) / 32;  // tabu words per lane (direct phase)
   constexpr int KW = (CP + H - 1) / H;
@@ -73,6 +201,15 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
   constexpr int K = KP < CP / 4 ? KP : CP / 4;
   using Parts = ChunkParts<CP, K>;
   constexpr int PP = (Parts::max_cities() + H - 1) / H;  // cities per lane in the rescan
+  constexpr int A = K > 1 ? 2 : 4;  // independent adders per part
+  constexpr int kPartDepth = (Parts::max_cities() + A - 1) / A + A - 1;
+  constexpr int kScan = H == 32 ? 5 : (H == 16 ? 4 : 3);
+  // roundings on the way to one side of the test: the lane's prefix (part
+  // sum, parts, scan, warps), the part's prefix inside the lane, the slot's
+  // prefix inside the part, the target and the differences; two to spare for
+  // the quantiser's floors and the second-order terms
+  constexpr int kRoundings = (kPartDepth + K + kScan + G) + (kPartDepth + K) + (PP + kScan) + 10;
+  constexpr float kEps = (float)kRoundings * 0x1p-24f;
   constexpr int kListCap = StageLayout<C, G, H>::kListEntries;
   const int n = I.n, ld = I.ld;
   const int hl = seg.hl;          // lane within the segment
@@ -133,7 +270,7 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
   for (; w.s < s_end; ++w.s) {
     const int s = w.s;
     const int cur = w.cur;
-    // Everyone is done with the previous row (the segment agreed on `cur`).
+    // Everyone is done with the previous row (the group agreed on `cur`).
     if (lane_copy) {
       const float4* src = reinterpret_cast<const float4*>(choice + (size_t)cur * ld);
       float4* dst = reinterpret_cast<float4*>(srow);
@@ -145,9 +282,9 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
     const int off = (s - 1) % H;
     if (off == 0) {
       const Philox4 x = step_draw(seed, (uint32_t)(s + hl), (uint32_t)ant, iter);
-      w.rwin = ((unsigned long long)x.x1 << 32) | x.x0;
+      w.u = __fmul_rn(__uint2float_rn(x.x1), 0x1p-32f);
     }
-    const unsigned long long r = seg.shfl(w.rwin, off);
+    const float u = seg.shfl(w.u, off);
     if (lane_copy) {
       group_wait();
     } else {
@@ -159,245 +296,183 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
     }
     const float* row = srow;
 
-    uint32_t v[CP];  // weight bits of the slots; w >= 0 orders like its bit pattern
+    // Sums of the open weights of each part (A independent adders a part).
+    float acc[K][A];
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int a = 0; a < A; ++a) acc[k][a] = 0.0f;
+#pragma unroll
+    for (int g = 0; g < CP / 4; ++g) {
+      int k = 0;
+#pragma unroll
+      for (int j = 1; j < K; ++j)
+        if (g >= Parts::first_group(j)) k = j;
+      float v[4];
+      if constexpr (!kGather) {
+        // Chunk entries at or beyond ld hold stale data; their tabu bits are set.
+        const float4 t = *reinterpret_cast<const float4*>(row + base + 4 * g);
+        v[0] = t.x;
+        v[1] = t.y;
+        v[2] = t.z;
+        v[3] = t.w;
+      } else {
+        const uint2 e = reinterpret_cast<const uint2*>(ulist + tg * CP)[g];
+        v[0] = __uint_as_float(entry_weight<kUnit>(row, e.x & 0xffffu));
+        v[1] = __uint_as_float(entry_weight<kUnit>(row, e.x >> 16));
+        v[2] = __uint_as_float(entry_weight<kUnit>(row, e.y & 0xffffu));
+        v[3] = __uint_as_float(entry_weight<kUnit>(row, e.y >> 16));
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int i = 4 * g + e;
+        bool open = true;
+        if constexpr (!kGather) open = !((vis[i >> 5] >> (i & 31)) & 1u);
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+          if (j == k && open) acc[j][e % A] = __fadd_rn(acc[j][e % A], v[e]);
+      }
+    }
+    // inclusive sums of the parts; the last is the thread's
+    float pincl[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      float v = acc[k][0];
+      if constexpr (A == 2) v = __fadd_rn(acc[k][0], acc[k][1]);
+      if constexpr (A == 4)
+        v = __fadd_rn(__fadd_rn(acc[k][0], acc[k][1]), __fadd_rn(acc[k][2], acc[k][3]));
+      pincl[k] = k ? __fadd_rn(pincl[k - 1], v) : v;
+    }
+    const float mine = pincl[K - 1];
+    const float incl = seg.inclusive_scan_f(mine);
+    const float wtot = seg.shfl(incl, H - 1);
+    float woff = 0.0f, S = wtot;
+    if constexpr (G > 1) {
+      if (hl == 0) gs->wtot[wg] = wtot;
+      group_wait();
+      S = 0.0f;
+#pragma unroll
+      for (int k = 0; k < G; ++k) {
+        if (k == wg) woff = S;
+        S = __fadd_rn(S, gs->wtot[k]);
+      }
+    }
+    // the target inside the warp, and inside this thread's range
+    const float t1 = __fsub_rn(__fmul_rn(u, S), woff);
+    const float err = S >= 0x1p-120f ? __fmul_rn(kEps, S) : __int_as_float(0x7f800000);
+    const int L = max(__ffs(seg.ballot(incl > t1)) - 1, 0);
+    const float t2 = seg.shfl(__fsub_rn(t1, __fsub_rn(incl, mine)), L);
+    // The part of lane L's slots that holds the target: every lane takes lane
+    // L's inclusive sums and decides alike.
+    int part = 0;
+    float t3 = t2;
+    if constexpr (K > 1) {
+      float before = 0.0f;
+#pragma unroll
+      for (int k = 0; k < K - 1; ++k) {
+        const float pk = seg.shfl(pincl[k], L);
+        if (pk <= t2) {
+          part = k + 1;
+          before = pk;
+        }
+      }
+      t3 = __fsub_rn(t2, before);
+    }
+    // The segment rescans that part, PP slots per lane.
+    const int pstart = 4 * (part * Parts::NG / K);
+    const int psz = 4 * ((part + 1) * Parts::NG / K) - pstart;
+    // lane L's tabu bits (direct phase; gather phases read them from the
+    // list: a visited slot reads weight 0)
+    uint32_t visL[kGather ? 1 : NW];
     if constexpr (!kGather) {
 #pragma unroll
-      for (int i = 0; i < CP; i += 4) {
-        const uint4 t = *reinterpret_cast<const uint4*>(row + base + i);
-        v[i] = t.x;
-        v[i + 1] = t.y;
-        v[i + 2] = t.z;
-        v[i + 3] = t.w;
-      }
-    } else {
-      const uint2* lw = reinterpret_cast<const uint2*>(ulist + tg * CP);
-#pragma unroll
-      for (int i = 0; i < CP; i += 4) {
-        const uint2 e = lw[i >> 2];
-        v[i] = entry_weight<kUnit>(row, e.x & 0xffffu);
-        v[i + 1] = entry_weight<kUnit>(row, e.x >> 16);
-        v[i + 2] = entry_weight<kUnit>(row, e.y & 0xffffu);
-        v[i + 3] = entry_weight<kUnit>(row, e.y >> 16);
-      }
+      for (int wd = 0; wd < NW; ++wd) visL[wd] = seg.shfl(vis[wd], L);
     }
-    // The max pass.  A float max equals the integer max of the bit patterns
-    // for weights >= 0 (no NaN; subnormals kept: no flush to zero); it
-    // measured faster in the compacted phases and for direct chunks of 44
-    // cities or more (n = 2392 0.6 %, n = 1002 0.45 %), slower for a direct
-    // chunk of 36 (0.6 %).
-    constexpr bool kFloatMax = kGather || C >= 44;
-    uint32_t mx;
-    if constexpr (kFloatMax) {
-      float m4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const int tL = wg * 32 + L;  // thread of lane L within the group
+    float wv[PP];
+    int cc[PP];
+    float ps = 0.0f;
 #pragma unroll
-      for (int i = 0; i < CP; ++i) {
-        if constexpr (!kGather) {
-          if ((vis[i >> 5] >> (i & 31)) & 1u) v[i] = 0u;
-        }
-        m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(v[i]));
-      }
-      mx = seg.max_u32(__float_as_uint(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]))));
-    } else {
-      uint32_t m4[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-      for (int i = 0; i < CP; ++i) {
-        if constexpr (!kGather) {
-          if ((vis[i >> 5] >> (i & 31)) & 1u) v[i] = 0u;
-        }
-        m4[i & 3] = max(m4[i & 3], v[i]);
-      }
-      mx = seg.max_u32(max(max(m4[0], m4[1]), max(m4[2], m4[3])));
-    }
-    if constexpr (G > 1) {
-      if (hl == 0) gs->wmax[wg] = mx;
-      group_wait();
-#pragma unroll
-      for (int k = 0; k < G; ++k) mx = max(mx, gs->wmax[k]);
-    }
-
-    int next;
-    int chosen = -1, chosen_slot = 0;  // gather phases: the thread and slot to mark
-    if (mx == 0u) {
-      // Every unvisited weight is zero: the lowest unvisited city.
-      uint32_t cand = 0xffffffffu;
+    for (int p = 0; p < PP; ++p) {
+      const int pi = hl * PP + p;  // position within the part
+      const int li = pstart + pi;  // slot within lane L's slots
+      float v = 0.0f;
+      int c = 0;
       if constexpr (!kGather) {
+        uint32_t word = FULL;
 #pragma unroll
-        for (int wd = NW - 1; wd >= 0; --wd) {
-          const uint32_t fr = ~vis[wd];
-          if (fr) cand = (uint32_t)(base + 32 * wd + __ffs(fr) - 1);
-        }
-      } else {
-        // the smallest entry: kZeroEntry is above every city's
-        const uint2* lw = reinterpret_cast<const uint2*>(ulist + tg * CP);
-#pragma unroll
-        for (int i = 0; i < CP; i += 4) {
-          const uint2 e = lw[i >> 2];
-          cand = min(cand, min(min(e.x & 0xffffu, e.x >> 16), min(e.y & 0xffffu, e.y >> 16)));
-        }
+        for (int wd = 0; wd < NW; ++wd)
+          if (wd == (li >> 5)) word = visL[wd];
+        c = tL * C + li;
+        if (pi < psz && !((word >> (li & 31)) & 1u)) v = row[c];
+      } else if (pi < psz) {
+        const uint32_t e = ulist[tL * CP + li];
+        v = __uint_as_float(entry_weight<kUnit>(row, e));
+        c = (int)(e / kUnit);
       }
-      cand = seg.min_u32(cand);
-      if constexpr (G > 1) {
-        if (hl == 0) gs->wmin[wg] = (int)cand;
-        group_wait();
-#pragma unroll
-        for (int k = 0; k < G; ++k) cand = min(cand, (uint32_t)gs->wmin[k]);
-      }
-      const uint32_t cand_entry = cand;  // gather phases: the list entry
-      if constexpr (kGather) cand /= kUnit;
-      next = (int)cand;
-      if constexpr (kGather) {
-        // the thread whose slot holds that city points the slot at the zero
-        // weight (no other thread reads the list until the step's end)
-#pragma unroll
-        for (int i = 0; i < CP; ++i)
-          if (ulist[tg * CP + i] == cand_entry) ulist[tg * CP + i] = (uint16_t)kZeroEntry;
-      }
+      cc[p] = c;
+      wv[p] = v;
+      ps = __fadd_rn(ps, v);
+    }
+    const float incl2 = seg.inclusive_scan_f(ps);
+    // The city whose interval holds the target with the error to spare (at
+    // most one slot of the segment).
+    const float hi_t = __fadd_rn(t3, err), lo_t = __fsub_rn(t3, err);
+    float c0 = __fsub_rn(incl2, ps);
+    int pick = -1;
+    if constexpr (PP == 1) {
+      if (incl2 > hi_t && c0 < lo_t) pick = 0;
     } else {
-      const int sc = kRouletteBits - 1 - exponent_of_bits(mx);
-      float f1, f1s, f2;
-      quant_factors(sc, f1, f1s, f2);
-      if (f2 != 1.0f) {
-#pragma unroll
-        for (int i = 0; i < CP; ++i) v[i] = __float_as_uint(__fmul_rn(__uint_as_float(v[i]), f2));
-      }
-      uint32_t phi[K], plo[K];
-      chunk_sum_parts<CP, K>(v, f1, f1s, phi, plo);
-      uint32_t hs = phi[0], ls = plo[0];
-#pragma unroll
-      for (int k = 1; k < K; ++k) {
-        hs += phi[k];
-        ls += plo[k];
-      }
-      // Inclusive sums of the thread's first K - 1 parts (they overlap the
-      // scan below; the selected lane's are used for the part choice).
-      unsigned long long pincl[K > 1 ? K - 1 : 1];
-      if constexpr (K > 1) {
-        pincl[0] = part_value<CP, K>(phi, plo, 0);
-#pragma unroll
-        for (int k = 1; k < K - 1; ++k) pincl[k] = pincl[k - 1] + part_value<CP, K>(phi, plo, k);
-      }
-      const uint32_t offb = (uint32_t)CP * kTwo23Bits;
-      const unsigned long long mine = ((unsigned long long)(hs - offb) << 23) + (ls - offb);
-      const unsigned long long incl = seg.inclusive_scan(mine);
-      const unsigned long long wtot = seg.shfl(incl, H - 1);
-      unsigned long long woff = 0, Q = wtot;
-      if constexpr (G > 1) {
-        if (hl == 0) gs->wsum[wg] = wtot;
-        group_wait();
-        Q = 0;
-#pragma unroll
-        for (int k = 0; k < G; ++k) {
-          const unsigned long long u = gs->wsum[k];
-          if (k < wg) woff += u;
-          Q += u;
-        }
-      }
-      const unsigned long long T = __umul64hi(r, Q);
-      // The warp whose range holds T finds the city (every warp when G = 1).
-      if (G == 1 || (T >= woff && T - woff < wtot)) {
-      const unsigned long long t1 = T - woff;
-      const int L = max(__ffs(seg.ballot(incl > t1)) - 1, 0);
-      const unsigned long long t2 = t1 - seg.shfl(incl - mine, L);
-      // The part of lane L's slots that holds the target: the first whose
-      // inclusive sum exceeds t2 (the sums ascend, so it is the count of
-      // those at most t2).  Every lane takes lane L's sums and decides alike.
-      int part = 0;
-      unsigned long long t3 = t2;
-      if constexpr (K > 1) {
-        unsigned long long before = 0;
-#pragma unroll
-        for (int k = 0; k < K - 1; ++k) {
-          const unsigned long long pk = seg.shfl(pincl[k], L);
-          if (pk <= t2) {
-            part = k + 1;
-            before = pk;
-          }
-        }
-        t3 = t2 - before;
-      }
-      // The segment rescans that part, PP slots per lane.
-      const int pstart = 4 * (part * Parts::NG / K);
-      const int psz = 4 * ((part + 1) * Parts::NG / K) - pstart;
-      // lane L's tabu bits (direct phase; gather phases read them from the
-      // list: a visited slot reads weight 0)
-      uint32_t visL[kGather ? 1 : NW];
-      if constexpr (!kGather) {
-#pragma unroll
-        for (int wd = 0; wd < NW; ++wd) visL[wd] = seg.shfl(vis[wd], L);
-      }
-      unsigned long long qv[PP];
-      int cc[PP];
-      unsigned long long ps = 0;
 #pragma unroll
       for (int p = 0; p < PP; ++p) {
-        const int pi = hl * PP + p;  // position within the part
-        const int li = pstart + pi;  // slot within lane L's slots
-        uint32_t w8 = 0u;
-        int c = 0;
-        const int tL = wg * 32 + L;  // thread of lane L within the group
-        if constexpr (!kGather) {
-          uint32_t word = FULL;
-#pragma unroll
-          for (int wd = 0; wd < NW; ++wd)
-            if (wd == (li >> 5)) word = visL[wd];
-          const bool open = pi < psz && !((word >> (li & 31)) & 1u);
-          c = (G > 1 ? tL : L) * C + li;
-          if (open && c < ld) w8 = __float_as_uint(row[c]);
-        } else {
-          if (pi < psz) {
-            const uint32_t e = ulist[(G > 1 ? tL : L) * CP + li];
-            w8 = entry_weight<kUnit>(row, e);
-            c = (int)(e / kUnit);
-          }
-        }
-        cc[p] = c;
-        qv[p] = quant_value(w8, f1, f1s, f2);
-        ps += qv[p];
+        const float c1 = p == PP - 1 ? incl2 : __fadd_rn(c0, wv[p]);
+        if (c1 > hi_t && c0 < lo_t) pick = p;
+        c0 = c1;
       }
-      const unsigned long long incl2 = seg.inclusive_scan(ps);
-      const int L2 = max(__ffs(seg.ballot(incl2 > t3)) - 1, 0);
-      int pick = 0;
-      if constexpr (PP > 1) {
-        if (hl == L2) {
-          unsigned long long c = incl2 - ps;
-          pick = -1;
-#pragma unroll
-          for (int p = 0; p < PP; ++p) {
-            c += qv[p];
-            if (pick < 0 && c > t3) pick = p;
-          }
-        }
-        pick = max(seg.shfl(pick, L2), 0);
-      }
-      int pc = cc[0];
+    }
+    const uint32_t sure = seg.ballot(pick >= 0);
+    const int L2 = max(__ffs(sure) - 1, 0);
+    int pc = cc[0];
+    if constexpr (PP > 1) {
 #pragma unroll
       for (int p = 1; p < PP; ++p)
         if (p == pick) pc = cc[p];
-      next = seg.shfl(pc, L2);
-      chosen = G > 1 ? wg * 32 + L : L;
-      chosen_slot = pstart + L2 * PP + pick;
-      if constexpr (G > 1) {
-        if (hl == 0) {
-          gs->next = next;
-          gs->wmin[0] = chosen;
-          gs->wmin[1] = chosen_slot;
-        }
-      }
-      }
-      if constexpr (G > 1) {
-        group_wait();
-        next = gs->next;
-        chosen = gs->wmin[0];
-        chosen_slot = gs->wmin[1];
-      }
+      pick = seg.shfl(pick, L2);
     }
+    Pick got{seg.shfl(pc, L2), tL, pstart + L2 * PP + (PP > 1 ? pick : 0)};
+    bool found = sure != 0u;
+    if constexpr (G > 1) {
+      // One warp at most is sure.  fnext[s & 1] was reset between the two
+      // barriers of the step before, after every read of step s - 2's.
+      if (found && hl == 0) {
+        gs->fnext[s & 1] = got.next;
+        gs->chosen = got.chosen;
+        gs->slot = got.slot;
+      }
+      if (tg == 0) gs->fnext[(s + 1) & 1] = -1;
+      group_wait();
+      got = Pick{gs->fnext[s & 1], gs->chosen, gs->slot};
+      found = got.next >= 0;
+    }
+    if (!found) {
+      const Philox4 x = step_draw(seed, (uint32_t)s, (uint32_t)ant, iter);
+      const unsigned long long r = ((unsigned long long)x.x1 << 32) | x.x0;
+      uint32_t v3[3] = {FULL, FULL, FULL};
+      if constexpr (!kGather) {
+#pragma unroll
+        for (int wd = 0; wd < NW; ++wd) v3[wd] = vis[wd];
+      }
+      got = exact_pick<G, H, kUnit>(row, kGather ? ulist : nullptr, CP, kZeroEntry, v3[0], v3[1],
+                                    v3[2], tg, bar_id, gs, r);
+    }
+    int next = got.next;
 
     // A city outside [0, n) can only come from a defect; record it and stay
     // in bounds instead of reading past the matrix.
     if ((unsigned)next >= (unsigned)n) {
       if (tg == 0) atomicOr(&I.st->status, kStatusBadTour);
       next = start;
-      chosen = -1;
+      got.chosen = -1;
     }
     if constexpr (!kGather) {
       const int li = next - base;
@@ -406,17 +481,23 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
         for (int wd = 0; wd < NW; ++wd)
           if (wd == (li >> 5)) vis[wd] |= 1u << (li & 31);
       }
-    } else if (tg == chosen) {
-      // every read of this entry in this step came before the shuffle that
-      // decided it
-      ulist[tg * CP + chosen_slot] = (uint16_t)kZeroEntry;
+    } else if (tg == got.chosen) {
+      // every read of this entry in this step came before the shuffle (or
+      // barrier) that decided it
+      ulist[tg * CP + got.slot] = (uint16_t)kZeroEntry;
     }
     if (tg == 0) tour[s] = next;
     w.cur = next;
-    group_wait();
+    // G > 1: the barrier above (or exact_pick's last) already follows every
+    // read of the row; the lanes of a warp still have to see the mark.
+    if (G > 1 && !lane_copy)
+      __syncwarp();
+    else
+      group_wait();
   }
 
   if constexpr (CPN > 0) {
+    if constexpr (G > 1) group_wait();
     // List the unvisited cities for the next phase, ascending: lane after
     // lane, each lane's slots in order.
     uint32_t cnt = 0;
@@ -446,9 +527,9 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
       total = 0;
 #pragma unroll
       for (int q = 0; q < G; ++q) {
-        const int u = (int)gs->wsum[q];
-        if (q < wg) k += u;
-        total += u;
+        const int v = (int)gs->wsum[q];
+        if (q < wg) k += v;
+        total += v;
       }
     }
     group_wait();  // the list of this phase is no longer read
@@ -520,10 +601,11 @@ __device__ __forceinline__ void construct_ant_phased(const Instance& I, const in
     mbar_init(bar, 1);
     fence_mbar_init();
     srow[StageLayout<C, G, H>::kZeroSlot] = 0.0f;  // the weight of a visited list slot
+    if (G > 1) gs->fnext[0] = gs->fnext[1] = -1;
   }
   group_wait();
 
-  WalkState w{start, 1, 0, 0ull, 0u, true};
+  WalkState w{start, 1, 0, 0.0f, 0u, true};
   eq1_phases<C, G, H, kPool, 0>(I, ant, tg, seg, gs, bar_id, srow, ulist, start, w, lane_copy);
   if (tg == 0) tour[n] = start;
   group_wait();
