@@ -881,15 +881,15 @@ __global__ void __launch_bounds__(256) construct_items_kernel(const Instance* __
 
 // The Eq. 1 walk with compaction (construct_phased.cuh), one group of H lanes
 // (or two warps) per ant.  Its phases are inlined into one body; without a
-// ceiling the register allocator adds their needs up instead of sharing them
-// (233 registers at C = 76, where phase 0 alone needs 128).  The ceilings were
-// chosen by measurement on the GB300: 128 from C = 44 (no spills); 72 at
-// C = 36 (no spills; the batched step 0.9 % faster than at 80, one instance
-// of n = 1002 the same); 64 up to C = 28 (the batched step 22.38 ms against
-// 22.91 ms at 80; 56 spills and was 2.5 % slower).
+// ceiling the register allocator hoists the row's loads.  The ceilings were
+// chosen by measurement on the GB300: 64 up to C = 36, where the shared
+// memory of a row leaves room for 32 ants an SM (n = 1002, m = 4864: 1.58 ms
+// against 1.98 at 72; a step of 256 instances 14.3 ms against 14.5; 48 and 56
+// are 1-2 % slower everywhere); above, the rows limit the ants and 128 costs
+// nothing (n = 2392 3.30 ms; 96: 3.32, 72: 3.34).
 template <int C>
 struct PhasedRegs {
-  static constexpr int v = C <= 28 ? 64 : (C <= 36 ? 72 : 128);
+  static constexpr int v = C <= 36 ? 64 : 128;
 };
 
 template <int C, int G, int H>

@@ -59,12 +59,13 @@ struct Pick {
 
 // The integer roulette of one step from the staged row (reading R2), slot by
 // slot: taken when the float search below cannot tell which city the target
-// falls on, or no open weight is positive.  A call of its own, so that it
-// costs the walk neither registers nor instructions (0.1-2 % of the steps).
+// falls on, or no open weight is positive (0.1-2 % of the steps).  Its loops
+// stay rolled and read the row again, so that it costs the walk no registers;
+// as a call of its own it cost 3 % (the values kept across the call).
 // list = nullptr: slot i of thread tg is city tg*cp + i with tabu bits v0..v2;
 // otherwise the list entry tg*cp + i.
 template <int G, int H, uint32_t kUnit>
-__device__ __noinline__ Pick exact_pick(const float* row, uint16_t* list, int cp, uint32_t zero_entry,
+__device__ __forceinline__ Pick exact_pick(const float* row, uint16_t* list, int cp, uint32_t zero_entry,
                                         uint32_t v0, uint32_t v1, uint32_t v2, int tg, int bar_id,
                                         GroupSmem* gs, unsigned long long r) {
   constexpr int NT = G * H;
@@ -82,7 +83,7 @@ __device__ __noinline__ Pick exact_pick(const float* row, uint16_t* list, int cp
     return (word >> (i & 31)) & 1u ? 0u : __float_as_uint(row[tg * cp + i]);
   };
   uint32_t mx = 0u;
-#pragma unroll 4
+#pragma unroll 1
   for (int i = 0; i < cp; ++i) mx = max(mx, weight(i));
   mx = seg.max_u32(mx);
   if constexpr (G > 1) {
@@ -95,7 +96,8 @@ __device__ __noinline__ Pick exact_pick(const float* row, uint16_t* list, int cp
     // Every open weight is zero: the lowest open city (a list's smallest
     // entry; zero_entry is above every city's).
     uint32_t cand = 0xffffffffu;
-    for (int i = cp - 1; i >= 0; --i) {
+  #pragma unroll 1
+  for (int i = cp - 1; i >= 0; --i) {
       if (list) {
         cand = min(cand, (uint32_t)list[tg * cp + i]);
       } else {
@@ -112,6 +114,7 @@ __device__ __noinline__ Pick exact_pick(const float* row, uint16_t* list, int cp
     }
     if (!list) return Pick{(int)cand, -1, 0};
     // no other thread reads these entries until the step's end
+#pragma unroll 1
     for (int i = 0; i < cp; ++i)
       if (list[tg * cp + i] == cand) list[tg * cp + i] = (uint16_t)zero_entry;
     return Pick{(int)(cand / kUnit), -1, 0};
@@ -119,7 +122,7 @@ __device__ __noinline__ Pick exact_pick(const float* row, uint16_t* list, int cp
   float f1, f1s, f2;
   quant_factors(kRouletteBits - 1 - exponent_of_bits(mx), f1, f1s, f2);
   unsigned long long mine = 0;
-#pragma unroll 4
+#pragma unroll 1
   for (int i = 0; i < cp; ++i) mine += quant_value(weight(i), f1, f1s, f2);
   const unsigned long long incl = seg.inclusive_scan(mine);
   const unsigned long long wtot = seg.shfl(incl, H - 1);
@@ -142,6 +145,7 @@ __device__ __noinline__ Pick exact_pick(const float* row, uint16_t* list, int cp
     int slot = 0, city = 0;
     if (hl == L) {
       unsigned long long c = woff + incl - mine;
+#pragma unroll 1
       for (; slot < cp - 1; ++slot) {
         c += quant_value(weight(slot), f1, f1s, f2);
         if (c > T) break;
@@ -183,32 +187,27 @@ __device__ __noinline__ Pick exact_pick(const float* row, uint16_t* list, int cp
 // target within the error of a boundary; S zero, tiny, infinite or NaN) the
 // step runs exact_pick().  This drops the max pass, the three FMAs of the
 // quantiser and half of every shuffle (64-bit scans) from a step.
-template <int C, int CP, int CPN, int G, int H, bool kGather, bool kPool>
+template <int C, int CP, int CPN, int G, int H, bool kGather, bool kPool, bool kLane>
 __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, const int tg,
                                           const Seg<H> seg, GroupSmem* gs, const int bar_id,
                                           float* srow, uint16_t* ulist, const int start,
-                                          const int s_end, WalkState& w, const bool lane_copy) {
+                                          const int s_end, WalkState& w) {
   static_assert(CP % 4 == 0 && CP >= 4 && CP <= 96, "CP must be a multiple of 4 in [4,96]");
   static_assert(kGather || CP == C, "the direct phase reads whole chunks");
   static_assert(G == 1 || H == 32, "several warps per ant use whole warps");
   constexpr int NT = G * H;  // threads per ant
   constexpr int NW = (CP + 31) / 32;  // tabu words per lane (direct phase)
-  constexpr int KW = (CP + H - 1) / H;
-  // parts of the thread's slots for the second-level search: one per 32
-  // slots (up to four); with the branch-free part choice a split pays for
-  // two words too (n = 1002: 1.138 to 1.126 ms)
-  constexpr int KP = KW < 4 ? KW : 4;
-  constexpr int K = KP < CP / 4 ? KP : CP / 4;
-  using Parts = ChunkParts<CP, K>;
-  constexpr int PP = (Parts::max_cities() + H - 1) / H;  // cities per lane in the rescan
-  constexpr int A = K > 1 ? 2 : 4;  // independent adders per part
-  constexpr int kPartDepth = (Parts::max_cities() + A - 1) / A + A - 1;
+  // The second-level search takes a part of kPart slots, whole in every lane.
+  constexpr int kPart = CP < 8 ? CP : 8;
+  constexpr int K = (CP + kPart - 1) / kPart;
+  constexpr bool kHalfTail = CP % kPart != 0;  // the last part holds four slots
   constexpr int kScan = H == 32 ? 5 : (H == 16 ? 4 : 3);
   // roundings on the way to one side of the test: the lane's prefix (part
-  // sum, parts, scan, warps), the part's prefix inside the lane, the slot's
-  // prefix inside the part, the target and the differences; two to spare for
-  // the quantiser's floors and the second-order terms
-  constexpr int kRoundings = (kPartDepth + K + kScan + G) + (kPartDepth + K) + (PP + kScan) + 10;
+  // sums of 4 + 1 additions, parts, scan, warps), the part's prefix inside
+  // the lane, the slot's prefix inside the part, the target and the
+  // differences; two to spare for the quantiser's floors and the second-order
+  // terms
+  constexpr int kRoundings = (5 + K + kScan + G) + (5 + K) + kPart + 10;
   constexpr float kEps = (float)kRoundings * 0x1p-24f;
   constexpr int kListCap = StageLayout<C, G, H>::kListEntries;
   const int n = I.n, ld = I.ld;
@@ -271,13 +270,17 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
     const int s = w.s;
     const int cur = w.cur;
     // Everyone is done with the previous row (the group agreed on `cur`).
-    if (lane_copy) {
-      const float4* src = reinterpret_cast<const float4*>(choice + (size_t)cur * ld);
-      float4* dst = reinterpret_cast<float4*>(srow);
-      for (int i = tg; i < (ld >> 2); i += NT) dst[i] = src[i];
-    } else if (tg == 0) {
-      fence_proxy_async_smem();
-      bulk_load(srow_a, choice + (size_t)cur * ld, row_bytes, bar);
+    // Its reads are complete and nothing but the copy engine writes it, so
+    // the copy needs no proxy fence.
+    if constexpr (kLane) {
+      const float* src = choice + (size_t)cur * ld + 4 * tg;
+#pragma unroll
+      for (int i = 0; i < C / 4; ++i)
+        cp_async16_if(4 * (tg + i * NT) < ld, srow_a + 16u * (uint32_t)(tg + i * NT),
+                      src + 4 * i * NT);
+      cp_async_wait_all();
+    } else {
+      bulk_load_if(tg == 0, srow_a, choice + (size_t)cur * ld, row_bytes, bar);
     }
     const int off = (s - 1) % H;
     if (off == 0) {
@@ -285,10 +288,10 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
       w.u = __fmul_rn(__uint2float_rn(x.x1), 0x1p-32f);
     }
     const float u = seg.shfl(w.u, off);
-    if (lane_copy) {
+    if constexpr (kLane) {
       group_wait();
     } else {
-      if (w.waits_ok && !mbar_wait_bounded(bar, w.parity)) {
+      if (!mbar_try_wait(bar, w.parity) && w.waits_ok && !mbar_wait_bounded(bar, w.parity)) {
         w.waits_ok = false;  // stale data from here on; the status word says so
         if (tg == 0) atomicOr(&I.st->status, kStatusTimeout);
       }
@@ -296,51 +299,37 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
     }
     const float* row = srow;
 
-    // Sums of the open weights of each part (A independent adders a part).
-    float acc[K][A];
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-      for (int a = 0; a < A; ++a) acc[k][a] = 0.0f;
-#pragma unroll
-    for (int g = 0; g < CP / 4; ++g) {
-      int k = 0;
-#pragma unroll
-      for (int j = 1; j < K; ++j)
-        if (g >= Parts::first_group(j)) k = j;
-      float v[4];
-      if constexpr (!kGather) {
-        // Chunk entries at or beyond ld hold stale data; their tabu bits are set.
-        const float4 t = *reinterpret_cast<const float4*>(row + base + 4 * g);
-        v[0] = t.x;
-        v[1] = t.y;
-        v[2] = t.z;
-        v[3] = t.w;
-      } else {
-        const uint2 e = reinterpret_cast<const uint2*>(ulist + tg * CP)[g];
-        v[0] = __uint_as_float(entry_weight<kUnit>(row, e.x & 0xffffu));
-        v[1] = __uint_as_float(entry_weight<kUnit>(row, e.x >> 16));
-        v[2] = __uint_as_float(entry_weight<kUnit>(row, e.y & 0xffffu));
-        v[3] = __uint_as_float(entry_weight<kUnit>(row, e.y >> 16));
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int i = 4 * g + e;
-        bool open = true;
-        if constexpr (!kGather) open = !((vis[i >> 5] >> (i & 31)) & 1u);
-#pragma unroll
-        for (int j = 0; j < K; ++j)
-          if (j == k && open) acc[j][e % A] = __fadd_rn(acc[j][e % A], v[e]);
-      }
-    }
-    // inclusive sums of the parts; the last is the thread's
+    // Inclusive sums of the open weights over the parts; the last is the
+    // thread's.
     float pincl[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      float v = acc[k][0];
-      if constexpr (A == 2) v = __fadd_rn(acc[k][0], acc[k][1]);
-      if constexpr (A == 4)
-        v = __fadd_rn(__fadd_rn(acc[k][0], acc[k][1]), __fadd_rn(acc[k][2], acc[k][3]));
+      float acc[2] = {0.0f, 0.0f};
+#pragma unroll
+      for (int g = k * (kPart / 4); g < (k + 1) * (kPart / 4) && g < CP / 4; ++g) {
+        float v[4];
+        if constexpr (!kGather) {
+          // Chunk entries at or beyond ld hold stale data; their tabu bits are set.
+          const float4 t = *reinterpret_cast<const float4*>(row + base + 4 * g);
+          v[0] = t.x;
+          v[1] = t.y;
+          v[2] = t.z;
+          v[3] = t.w;
+        } else {
+          const uint2 e = reinterpret_cast<const uint2*>(ulist + tg * CP)[g];
+          v[0] = __uint_as_float(entry_weight<kUnit>(row, e.x & 0xffffu));
+          v[1] = __uint_as_float(entry_weight<kUnit>(row, e.x >> 16));
+          v[2] = __uint_as_float(entry_weight<kUnit>(row, e.y & 0xffffu));
+          v[3] = __uint_as_float(entry_weight<kUnit>(row, e.y >> 16));
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          bool open = true;
+          if constexpr (!kGather) open = !((vis[(4 * g + e) >> 5] >> ((4 * g + e) & 31)) & 1u);
+          if (open) acc[e & 1] = __fadd_rn(acc[e & 1], v[e]);
+        }
+      }
+      const float v = __fadd_rn(acc[0], acc[1]);
       pincl[k] = k ? __fadd_rn(pincl[k - 1], v) : v;
     }
     const float mine = pincl[K - 1];
@@ -357,90 +346,85 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
         S = __fadd_rn(S, gs->wtot[k]);
       }
     }
-    // the target inside the warp, and inside this thread's range
+    // The target inside this thread's range, and the part of the thread's
+    // slots that holds it if it lies there.  Every lane works this out while
+    // the vote finds the lane.
     const float t1 = __fsub_rn(__fmul_rn(u, S), woff);
     const float err = S >= 0x1p-120f ? __fmul_rn(kEps, S) : __int_as_float(0x7f800000);
-    const int L = max(__ffs(seg.ballot(incl > t1)) - 1, 0);
-    const float t2 = seg.shfl(__fsub_rn(t1, __fsub_rn(incl, mine)), L);
-    // The part of lane L's slots that holds the target: every lane takes lane
-    // L's inclusive sums and decides alike.
-    int part = 0;
-    float t3 = t2;
-    if constexpr (K > 1) {
-      float before = 0.0f;
+    const uint32_t passed = seg.ballot(!(incl > t1));
+    const float t2 = __fsub_rn(t1, __fsub_rn(incl, mine));
+    uint32_t part = 0u;
+    float before = 0.0f;
 #pragma unroll
-      for (int k = 0; k < K - 1; ++k) {
-        const float pk = seg.shfl(pincl[k], L);
-        if (pk <= t2) {
-          part = k + 1;
-          before = pk;
-        }
+    for (int k = 0; k < K - 1; ++k)
+      if (pincl[k] <= t2) {
+        part = (uint32_t)(k + 1);
+        before = pincl[k];
       }
-      t3 = __fsub_rn(t2, before);
-    }
-    // The segment rescans that part, PP slots per lane.
-    const int pstart = 4 * (part * Parts::NG / K);
-    const int psz = 4 * ((part + 1) * Parts::NG / K) - pstart;
-    // lane L's tabu bits (direct phase; gather phases read them from the
-    // list: a visited slot reads weight 0)
-    uint32_t visL[kGather ? 1 : NW];
     if constexpr (!kGather) {
+      // the part's tabu bits beside its number
+      uint32_t word = vis[0];
 #pragma unroll
-      for (int wd = 0; wd < NW; ++wd) visL[wd] = seg.shfl(vis[wd], L);
+      for (int wd = 1; wd < NW; ++wd)
+        if (part * kPart >= 32u * wd) word = vis[wd];
+      part |= (word >> ((part * kPart) & 31u)) << 8;
     }
-    const int tL = wg * 32 + L;  // thread of lane L within the group
-    float wv[PP];
-    int cc[PP];
-    float ps = 0.0f;
-#pragma unroll
-    for (int p = 0; p < PP; ++p) {
-      const int pi = hl * PP + p;  // position within the part
-      const int li = pstart + pi;  // slot within lane L's slots
-      float v = 0.0f;
-      int c = 0;
-      if constexpr (!kGather) {
-        uint32_t word = FULL;
-#pragma unroll
-        for (int wd = 0; wd < NW; ++wd)
-          if (wd == (li >> 5)) word = visL[wd];
-        c = tL * C + li;
-        if (pi < psz && !((word >> (li & 31)) & 1u)) v = row[c];
-      } else if (pi < psz) {
-        const uint32_t e = ulist[tL * CP + li];
-        v = __uint_as_float(entry_weight<kUnit>(row, e));
-        c = (int)(e / kUnit);
-      }
-      cc[p] = c;
-      wv[p] = v;
-      ps = __fadd_rn(ps, v);
-    }
-    const float incl2 = seg.inclusive_scan_f(ps);
-    // The city whose interval holds the target with the error to spare (at
-    // most one slot of the segment).
+    // the inclusive sums ascend: as many lanes are passed as lie before L
+    const int L = min(__popc(passed), H - 1);
+    const float t3 = seg.shfl(__fsub_rn(t2, before), L);
+    part = seg.shfl(part, L);
+    const uint32_t closed = part >> 8;  // direct phase
+    if constexpr (!kGather) part &= 0xffu;
+    // The slot inside the part: every lane reads the part and decides alike,
+    // with no further exchange.
     const float hi_t = __fadd_rn(t3, err), lo_t = __fsub_rn(t3, err);
-    float c0 = __fsub_rn(incl2, ps);
-    int pick = -1;
-    if constexpr (PP == 1) {
-      if (incl2 > hi_t && c0 < lo_t) pick = 0;
-    } else {
+    const int tL = wg * 32 + L;  // thread of lane L within the group
+    const int pstart = (int)part * kPart;
+    float wv[kPart];
+    uint32_t ent[kGather ? kPart : 1] = {};
+    if constexpr (!kGather) {
+      // (past the chunk's end: the tabu bits there are set, and the staged row
+      // is followed by its mbarrier and the zero weight, 16 bytes)
+      const float4* p4 = reinterpret_cast<const float4*>(row + tL * C + pstart);
 #pragma unroll
-      for (int p = 0; p < PP; ++p) {
-        const float c1 = p == PP - 1 ? incl2 : __fadd_rn(c0, wv[p]);
-        if (c1 > hi_t && c0 < lo_t) pick = p;
-        c0 = c1;
+      for (int g = 0; g < kPart / 4; ++g) {
+        const float4 t = p4[g];
+        wv[4 * g] = t.x;
+        wv[4 * g + 1] = t.y;
+        wv[4 * g + 2] = t.z;
+        wv[4 * g + 3] = t.w;
+      }
+    } else {
+      const uint2* lw = reinterpret_cast<const uint2*>(ulist + tL * CP + pstart);
+      const bool half = kHalfTail && part == (uint32_t)(K - 1);
+#pragma unroll
+      for (int g = 0; g < kPart / 4; ++g) {
+        uint2 e = lw[g > 0 && half ? 0 : g];
+        if (g > 0 && half) e = make_uint2(kZeroEntry * 0x10001u, kZeroEntry * 0x10001u);
+        ent[4 * g] = e.x & 0xffffu;
+        ent[4 * g + 1] = e.x >> 16;
+        ent[4 * g + 2] = e.y & 0xffffu;
+        ent[4 * g + 3] = e.y >> 16;
+      }
+#pragma unroll
+      for (int i = 0; i < kPart; ++i) wv[i] = __uint_as_float(entry_weight<kUnit>(row, ent[i]));
+    }
+    // The first slot whose inclusive sum passes the target by the error; sure
+    // if the sum before it lies below the target by the error as well.
+    int slot = 0;
+    float c = 0.0f, below = 0.0f;
+    uint32_t hit = kGather ? ent[0] : 0u;
+#pragma unroll
+    for (int i = 0; i < kPart; ++i) {
+      if (kGather || !((closed >> i) & 1u)) c = __fadd_rn(c, wv[i]);
+      if (!(c > hi_t)) {
+        slot = i + 1;
+        below = c;
+        if (kGather && i + 1 < kPart) hit = ent[i + 1];
       }
     }
-    const uint32_t sure = seg.ballot(pick >= 0);
-    const int L2 = max(__ffs(sure) - 1, 0);
-    int pc = cc[0];
-    if constexpr (PP > 1) {
-#pragma unroll
-      for (int p = 1; p < PP; ++p)
-        if (p == pick) pc = cc[p];
-      pick = seg.shfl(pick, L2);
-    }
-    Pick got{seg.shfl(pc, L2), tL, pstart + L2 * PP + (PP > 1 ? pick : 0)};
-    bool found = sure != 0u;
+    bool found = slot < kPart && below < lo_t;
+    Pick got{kGather ? (int)(hit / kUnit) : tL * C + pstart + slot, tL, pstart + slot};
     if constexpr (G > 1) {
       // One warp at most is sure.  fnext[s & 1] was reset between the two
       // barriers of the step before, after every read of step s - 2's.
@@ -464,16 +448,15 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
       }
       got = exact_pick<G, H, kUnit>(row, kGather ? ulist : nullptr, CP, kZeroEntry, v3[0], v3[1],
                                     v3[2], tg, bar_id, gs, r);
+      // A city outside [0, n) can only come from a defect; record it and stay
+      // in bounds instead of reading past the matrix.
+      if ((unsigned)got.next >= (unsigned)n) {
+        if (tg == 0) atomicOr(&I.st->status, kStatusBadTour);
+        got.next = start;
+        got.chosen = -1;
+      }
     }
-    int next = got.next;
-
-    // A city outside [0, n) can only come from a defect; record it and stay
-    // in bounds instead of reading past the matrix.
-    if ((unsigned)next >= (unsigned)n) {
-      if (tg == 0) atomicOr(&I.st->status, kStatusBadTour);
-      next = start;
-      got.chosen = -1;
-    }
+    const int next = got.next;
     if constexpr (!kGather) {
       const int li = next - base;
       if (li >= 0 && li < C) {
@@ -490,7 +473,7 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
     w.cur = next;
     // G > 1: the barrier above (or exact_pick's last) already follows every
     // read of the row; the lanes of a warp still have to see the mark.
-    if (G > 1 && !lane_copy)
+    if constexpr (G > 1 && !kLane)
       __syncwarp();
     else
       group_wait();
@@ -554,20 +537,19 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
 // Phase J of the walk and the ones after it.  Phase J runs while the
 // unvisited cities do not fit in the next phase's slots, then lists them for
 // it; the last phase runs to the end of the tour.
-template <int C, int G, int H, bool kPool, int J>
+template <int C, int G, int H, bool kPool, bool kLane, int J>
 __device__ __forceinline__ void eq1_phases(const Instance& I, const int ant, const int tg,
                                            const Seg<H> seg, GroupSmem* gs, const int bar_id,
                                            float* srow, uint16_t* ulist, const int start,
-                                           WalkState& w, const bool lane_copy) {
+                                           WalkState& w) {
   using Cm = Compaction<C, G>;
   constexpr int CP = Cm::slots(J);
   constexpr int CPN = Cm::slots(J + 1);
   const int s_end = CPN > 0 ? max(w.s, I.n - G * H * CPN) : I.n;
-  eq1_phase<C, CP, CPN, G, H, (J > 0), kPool>(I, ant, tg, seg, gs, bar_id, srow, ulist, start,
-                                              s_end, w, lane_copy);
+  eq1_phase<C, CP, CPN, G, H, (J > 0), kPool, kLane>(I, ant, tg, seg, gs, bar_id, srow, ulist,
+                                                     start, s_end, w);
   if constexpr (CPN > 0)
-    eq1_phases<C, G, H, kPool, J + 1>(I, ant, tg, seg, gs, bar_id, srow, ulist, start, w,
-                                      lane_copy);
+    eq1_phases<C, G, H, kPool, kLane, J + 1>(I, ant, tg, seg, gs, bar_id, srow, ulist, start, w);
 }
 
 // The whole walk of one ant (G warps or one H-lane segment) and its length
@@ -606,7 +588,10 @@ __device__ __forceinline__ void construct_ant_phased(const Instance& I, const in
   group_wait();
 
   WalkState w{start, 1, 0, 0.0f, 0u, true};
-  eq1_phases<C, G, H, kPool, 0>(I, ant, tg, seg, gs, bar_id, srow, ulist, start, w, lane_copy);
+  if (lane_copy)
+    eq1_phases<C, G, H, kPool, true, 0>(I, ant, tg, seg, gs, bar_id, srow, ulist, start, w);
+  else
+    eq1_phases<C, G, H, kPool, false, 0>(I, ant, tg, seg, gs, bar_id, srow, ulist, start, w);
   if (tg == 0) tour[n] = start;
   group_wait();
 
