@@ -202,12 +202,12 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
   constexpr int K = (CP + kPart - 1) / kPart;
   constexpr bool kHalfTail = CP % kPart != 0;  // the last part holds four slots
   constexpr int kScan = H == 32 ? 5 : (H == 16 ? 4 : 3);
-  // roundings on the way to one side of the test: the lane's prefix (part
-  // sums of 4 + 1 additions, parts, scan, warps), the part's prefix inside
-  // the lane, the slot's prefix inside the part, the target and the
-  // differences; two to spare for the quantiser's floors and the second-order
-  // terms
-  constexpr int kRoundings = (5 + K + kScan + G) + (5 + K) + kPart + 10;
+  // roundings on the way to one side of the test: the prefix before the lane
+  // and, inside the target, S (part sums of 4 + 1 additions, parts, scan,
+  // warps each); the part's prefix inside the lane, the slot's prefix inside
+  // the part; the target and the differences; two to spare for the
+  // quantiser's floors and the second-order terms
+  constexpr int kRoundings = 2 * (5 + K + kScan + G) + (5 + K) + kPart + 10;
   constexpr float kEps = (float)kRoundings * 0x1p-24f;
   constexpr int kListCap = StageLayout<C, G, H>::kListEntries;
   const int n = I.n, ld = I.ld;
