@@ -488,13 +488,9 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
     }
     const float* row = srow;
 
-    // The race over long chunks reads its weights from the staged row as it
-    // goes (a register copy of 60 or more weights beside its per-candidate
-    // arithmetic measured slower); everything else works on a register copy.
-    constexpr bool kRowRace = R == 2 && C >= 60;
-    uint32_t v[C];  // weight bits; w >= 0 orders like its bit pattern
+    uint32_t v[R == 0 ? C : 1];  // weight bits; w >= 0 orders like its bit pattern
     uint32_t mx = 0u;
-    if constexpr (!kRowRace) {
+    if constexpr (R == 0) {
 #pragma unroll
       for (int i = 0; i < C; i += 4) {
         // Chunk entries at or beyond ld hold stale data; their tabu bits are set.
@@ -504,8 +500,6 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
         v[i + 2] = t.z;
         v[i + 3] = t.w;
       }
-    }
-    if constexpr (R != 2) {
       uint32_t m4[4] = {0u, 0u, 0u, 0u};  // four independent max chains
 #pragma unroll
       for (int i = 0; i < C; ++i) {
@@ -522,105 +516,139 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
     }
 
     int next;
+    // A group of four consecutive cities (C and base are multiples of 4)
+    // shares one Philox call.
+    auto group_draw = [&](int g) {
+      return philox4x32_10((uint32_t)s, (uint32_t)ant, iter, 1u + (uint32_t)((base >> 2) + g),
+                           (uint32_t)seed, (uint32_t)(seed >> 32));
+    };
+    // its weight bits, 0 where visited (entries at or beyond ld hold stale
+    // data; their tabu bits are set)
+    auto group_weights = [&](int g, uint32_t (&wv)[4]) {
+      const uint4 t = *reinterpret_cast<const uint4*>(row + base + 4 * g);
+      uint32_t word = vis[0];
+#pragma unroll
+      for (int w = 1; w < NW; ++w)
+        if (w == (g >> 3)) word = vis[w];
+      word >>= (4 * g) & 31;
+      wv[0] = word & 1u ? 0u : t.x;
+      wv[1] = word & 2u ? 0u : t.y;
+      wv[2] = word & 4u ? 0u : t.z;
+      wv[3] = word & 8u ? 0u : t.w;
+    };
     if constexpr (R == 1) {
-      // Scores u_j * w_j; a thread's four consecutive cities share one
-      // Philox call (C and base are multiples of 4).
-      // Each thread walks its cities in ascending order and keeps the first
-      // of its highest scores (bits of a non-negative float order like its
-      // value; 0 = no positive score); the segment reduction breaks ties by
-      // index.
-      uint32_t bs = 0u, bj = 0xffffffffu;
+      // Scores fl(u_j w_j), u_j <= 1: a score is at most its weight, so a
+      // group whose largest open weight is below the best score so far needs
+      // no random numbers.  Every lane starts with its heaviest group, the
+      // warp's best score then leaves a few groups in a few lanes.  (Drawing
+      // for every city took 788e6 warp-instructions at n = 1002 and 1.74 ms.)
+      constexpr int NGC = C / 4;
+      uint32_t gm[NGC];  // largest open weight of each group
+      uint32_t top = 0u, rem = 0u;
+      int g = 0;
 #pragma unroll
-      for (int i = 0; i < C; i += 4) {
-        const Philox4 x = philox4x32_10((uint32_t)s, (uint32_t)ant, iter,
-                                        1u + (uint32_t)((base + i) >> 2), (uint32_t)seed,
-                                        (uint32_t)(seed >> 32));
-        const uint32_t xs[4] = {x.x0, x.x1, x.x2, x.x3};
+      for (int i = 0; i < NGC; ++i) {
+        uint32_t wv[4];
+        group_weights(i, wv);
+        gm[i] = max(max(wv[0], wv[1]), max(wv[2], wv[3]));
+        if (gm[i] > top) {
+          top = gm[i];
+          g = i;
+        }
+        rem |= gm[i] ? 1u << i : 0u;
+      }
+      uint32_t bs = 0u, bj = 0xffffffffu, best = 0u;  // score bits order like scores
+      bool mine = NGC == 1 || rem != 0u;
+      do {
+        if (mine) {
+          const Philox4 x = group_draw(g);
+          const uint32_t xs[4] = {x.x0, x.x1, x.x2, x.x3};
+          uint32_t wv[4];
+          group_weights(g, wv);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const uint32_t sb = __float_as_uint(
-              __fmul_rn(candidate_uniform_of(xs[e]), __uint_as_float(v[i + e])));
-          if (sb > bs) {
-            bs = sb;
-            bj = (uint32_t)(base + i + e);
+          for (int e = 0; e < 4; ++e) {
+            const uint32_t sb =
+                __float_as_uint(__fmul_rn(candidate_uniform_of(xs[e]), __uint_as_float(wv[e])));
+            const uint32_t j = (uint32_t)(base + 4 * g + e);
+            if (sb > bs || (sb == bs && sb != 0u && j < bj)) {
+              bs = sb;
+              bj = j;
+            }
           }
+          rem &= ~(1u << g);
         }
-      }
+        best = seg.max_u32(bs);
 #pragma unroll
-      for (int o = H / 2; o > 0; o >>= 1) {
-        const uint32_t os = seg.shfl_xor(bs, o), oj = seg.shfl_xor(bj, o);
-        if (os > bs || (os == bs && oj < bj)) {
-          bs = os;
-          bj = oj;
-        }
-      }
+        for (int i = 0; i < NGC; ++i)
+          if (gm[i] < best) rem &= ~(1u << i);
+        mine = rem != 0u;
+        g = __ffs(rem) - 1;
+      } while (NGC > 1 && seg.ballot(mine));
+      bj = seg.min_u32(bs == best ? bj : 0xffffffffu);
       // (score bits << 32) | ~index: max = best score, lowest index
-      uint64_t key = bs ? ((uint64_t)bs << 32) | (uint32_t)(0xffffffffu - bj) : 0ull;
+      uint64_t key = best ? ((uint64_t)best << 32) | (uint32_t)(0xffffffffu - bj) : 0ull;
       if (G > 1) {
         if (hl == 0) gs->wsum[wg] = key;
         group_sync(bar_id, NT);
 #pragma unroll
         for (int w = 0; w < G; ++w) key = gs->wsum[w] > key ? gs->wsum[w] : key;
       }
-      if (key != 0) mx = 1u;  // a positive score exists
-      else mx = 0u;           // every score is 0: the rule below takes the lowest unvisited
+      mx = key != 0 ? 1u : 0u;  // 0: every score is 0, the lowest unvisited city
       next = (int)(0xffffffffu - (uint32_t)key);
     }
     if constexpr (R == 2) {
-      // Keys are non-negative floats (their bits order like their values);
-      // a visited city keeps the sentinel above every key.  A thread's four
-      // consecutive cities share one Philox call, and each thread walks its
-      // cities in ascending order keeping the first smallest key.
-      uint32_t bkey = 0xffffffffu, bj = 0xffffffffu;
-#pragma unroll
-      for (int i = 0; i < C; i += 4) {
-        const Philox4 x = philox4x32_10((uint32_t)s, (uint32_t)ant, iter,
-                                        1u + (uint32_t)((base + i) >> 2), (uint32_t)seed,
-                                        (uint32_t)(seed >> 32));
+      // Keys fl(E_j / w_j); non-negative floats order like their bits.  Since
+      // E = -ln u >= 1 - u, a city's key can only be below the best so far if
+      // 1 - u <= best w, a conversion and a multiply-add on the random word x
+      // (u = (floor(x / 2^8) + 1) 2^-24, so 1 - u >= 1 - (x + 256) 2^-32; the
+      // slack of 2048 in 2^32 and 2^-18 of best covers that, the roundings and
+      // E's 2.5 ulp).  Only cities that pass get the logarithm and the
+      // division.  Best keys below 2^-92 count as 2^-92: heavier weights than
+      // 2^92 pass, whatever underflows.  (The logarithm and division for
+      // every open city took 2.58e9 warp-instructions at n = 1002, 6.29 ms.)
+      constexpr uint32_t kInf = 0x7f800000u;
+      uint32_t bkey = kInf, bj = 0xffffffffu;  // the lane's smallest key and its city
+      float reach = __uint_as_float(kInf);     // best 2^32 (1 + 2^-18) over the warp
+#pragma unroll 3
+      for (int g = 0; g < C / 4; ++g) {
+        const Philox4 x = group_draw(g);
         const uint32_t xs[4] = {x.x0, x.x1, x.x2, x.x3};
         uint32_t wv[4];
-        if constexpr (kRowRace) {
-          const uint4 t = *reinterpret_cast<const uint4*>(row + base + i);
-          wv[0] = t.x;
-          wv[1] = t.y;
-          wv[2] = t.z;
-          wv[3] = t.w;
-        } else {
+        group_weights(g, wv);
+        uint32_t pass = 0u;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) wv[e] = v[i + e];
-        }
-        // the four tabu bits of these cities (i % 4 == 0: one word)
-        const uint32_t vis4 = vis[i >> 5] >> (i & 31);
+        for (int e = 0; e < 4; ++e)
+          if (__uint2float_rn(xs[e]) >= __fmaf_rn(-reach, __uint_as_float(wv[e]), 4294965248.0f))
+            pass |= 1u << e;
+        if (seg.ballot(pass != 0u)) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int li = i + e;
-          const float w = __uint_as_float(wv[e]);
-          const bool open = !((vis4 >> e) & 1u);
-          // visited cities skip the logarithm and the division
-          const float key = open && w > 0.0f ? __fdiv_rn(race_exponential(xs[e]), w)
-                                             : __uint_as_float(0x7f800000u);
-          const uint32_t kb = __float_as_uint(key);
-          if (open && kb < bkey) {
-            bkey = kb;
-            bj = (uint32_t)(base + li);
+          for (int e = 0; e < 4; ++e) {
+            const float w = __uint_as_float(wv[e]);
+            if (((pass >> e) & 1u) && w > 0.0f) {
+              const uint32_t kb = __float_as_uint(__fdiv_rn(race_exponential(xs[e]), w));
+              if (kb < bkey) {
+                bkey = kb;
+                bj = (uint32_t)(base + 4 * g + e);
+              }
+            }
           }
+          reach = fmaxf(__fmul_rn(__uint_as_float(seg.min_u32(bkey)), 4294983680.0f), 0x1p-60f);
         }
       }
-      uint64_t key = ((uint64_t)bkey << 32) | bj;
-#pragma unroll
-      for (int o = H / 2; o > 0; o >>= 1) {
-        const uint64_t other = seg.shfl_xor(key, o);
-        key = other < key ? other : key;
-      }
+      const uint32_t best = seg.min_u32(bkey);
+      bj = seg.min_u32(bkey == best ? bj : 0xffffffffu);
+      uint64_t key = ((uint64_t)best << 32) | bj;
       if (G > 1) {
         if (hl == 0) gs->wsum[wg] = key;
         group_sync(bar_id, NT);
 #pragma unroll
         for (int w = 0; w < G; ++w) key = gs->wsum[w] < key ? gs->wsum[w] : key;
       }
+      // no finite key: zero weights and overflowing keys are all +inf
+      mx = (uint32_t)(key >> 32) < kInf ? 1u : 0u;
       next = (int)(uint32_t)key;
     }
-    if ((R == 1 && mx != 0u) || R == 2) {
+    if (R != 0 && mx != 0u) {
       // chosen above
     } else if (mx == 0u) {
       // Every unvisited weight is zero: the lowest-index unvisited city.
