@@ -1,31 +1,20 @@
-// Tour construction (Section II, Eq. 1; data-parallel design of Section III-A).
+// Tour construction (Section II, Eq. 1; data-parallel design of Section III-A):
+// the pieces shared by the construction kernels, the per-candidate rules, and
+// the kernels.  The Eq. 1 walk itself is in construct_phased.cuh.
 //
 // One group of threads builds one ant's tour: G whole warps (H = 32), or an
 // H-lane segment of a warp (H = 8 or 16, G = 1), so that 32/H ants share
 // every warp instruction.  Thread t of the group owns the contiguous cities
-// [t*C, t*C + C) of every row: it reads them from the row staged in shared
-// memory into registers, keeps their tabu bits (the paper's "1 = unvisited"
-// integer per city, here one bit per city in registers) and takes part in the
-// selection.  Each step:
-//   1. one thread copies row choice[cur] into shared memory with the
-//      bulk-copy engine; the group waits on an mbarrier and reads its chunks
-//      (C floats per thread, conflict-free 16-byte loads); visited cities
-//      are zeroed;
-//   2. M = max over unvisited (max on the float bit patterns, which order
-//      like the values for w >= 0), across warps through shared memory;
-//   3. q_j = floor(w_j * 2^(45-ilogb M)) split exactly into two 23-bit halves
-//      by three round-toward-zero FP32 FMAs (FP32 pipe; no float-to-int
-//      conversion), per-thread u64 sums, warp inclusive scan, group totals
-//      -> Q;
-//   4. T = floor(r Q / 2^64) with r from Philox (one Philox call per lane per
-//      H steps, broadcast by shuffle);
-//   5. the thread whose prefix range holds T is found by ballot; it finds
-//      the part of its chunk (up to four parts of whole 4-city groups, from
-//      per-part sums kept in step 3) that holds the target, which is
-//      rescanned by all lanes of its warp segment (about one city each); a
-//      second scan and ballot give the city.
-// Every operation is an exact max or an exact integer sum, so the chosen city
-// is the same for every (C, G, H) tiling and equals the CPU oracle's choice.
+// [t*C, t*C + C) of every row, and keeps their tabu bits (the paper's "1 =
+// unvisited" integer per city, here one bit per city in registers).  At each
+// step one thread copies row choice[cur] into shared memory with the
+// bulk-copy engine; the group waits on an mbarrier, reads its chunks (C
+// floats per thread, conflict-free 16-byte loads) and selects.
+// The selection is defined by exact maxima and exact integer sums (the integer
+// roulette: M = max over unvisited; q_j = floor(w_j * 2^(45-ilogb M)); Q their
+// sum; T = floor(r Q / 2^64) with r from Philox; the first j whose prefix sum
+// exceeds T), so the chosen city is the same for every (C, G, H) tiling and
+// equals the CPU oracle's choice.
 // Every warp-level intrinsic names only the segment's lanes, so segments of
 // one warp never wait on each other even when their control flow differs.
 // After the last step the group computes C^k = sum of d over the tour and
@@ -42,8 +31,7 @@ struct GroupSmem {
   unsigned long long wsum[4];
   long long wlen[4];
   int wmin[4];
-  int next;
-  // the walk with compaction
+  // the Eq. 1 walk
   float wtot[4];
   int fnext[2], chosen, slot;
   int xnext, xchosen, xslot;
@@ -109,119 +97,6 @@ __device__ __forceinline__ void quant_factors(int sc, float& f1, float& f1s, flo
     f1s = pow2f(127);
     f2 = pow2f(e - 104);
   }
-}
-
-// Sum of q over the thread's C weights (already scaled by f2, see the
-// caller).  The float bit patterns are summed modulo 2^32 (two per IADD3)
-// and the C offsets of 0x4b000000 removed once; the true part sums are below
-// C * 2^23 <= 2^30, so the wrap-around is exact.
-template <int C>
-__device__ __forceinline__ unsigned long long chunk_sum(const uint32_t (&v)[C], float f1,
-                                                        float f1s) {
-  uint32_t hi0 = 0, lo0 = 0, hi1 = 0, lo1 = 0;
-#pragma unroll
-  for (int i = 0; i < C; i += 4) {
-    const QuantParts a = quant_parts(v[i], f1, f1s), b = quant_parts(v[i + 1], f1, f1s);
-    const QuantParts c = quant_parts(v[i + 2], f1, f1s), d = quant_parts(v[i + 3], f1, f1s);
-    hi0 += a.hi_bits + b.hi_bits;
-    lo0 += a.lo_bits + b.lo_bits;
-    hi1 += c.hi_bits + d.hi_bits;
-    lo1 += c.lo_bits + d.lo_bits;
-  }
-  const uint32_t off = (uint32_t)C * kTwo23Bits;
-  const uint32_t hi = hi0 + hi1 - off, lo = lo0 + lo1 - off;
-  return ((unsigned long long)hi << 23) + lo;
-}
-
-// A lane's chunk split into K parts of whole 4-city groups: part k holds the
-// groups [k*NG/K, (k+1)*NG/K), NG = C/4.  After the warp has found the lane
-// whose range holds the target, that lane finds the part from these sums,
-// and only the part's cities are searched city by city.
-template <int C, int K>
-struct ChunkParts {
-  static constexpr int NG = C / 4;
-  static_assert(K >= 1 && K <= NG, "1 <= K <= C/4 parts");
-  __host__ __device__ static constexpr int first_group(int k) { return k * NG / K; }
-  __host__ __device__ static constexpr int cities(int k) {
-    return 4 * (first_group(k + 1) - first_group(k));
-  }
-  static constexpr int max_cities() { return 4 * ((NG + K - 1) / K); }
-};
-
-// Per-part sums of q over the thread's C weights (already scaled by f2),
-// as hi/lo bit-pattern sums with their offsets still in (removed by
-// part_value).  Parts accumulate independently; a single part uses two
-// chains so that the adds still overlap.
-template <int C, int K>
-__device__ __forceinline__ void chunk_sum_parts(const uint32_t (&v)[C], float f1, float f1s,
-                                                uint32_t (&phi)[K], uint32_t (&plo)[K]) {
-  using Pt = ChunkParts<C, K>;
-  uint32_t hi2 = 0, lo2 = 0;  // second chain of a single part
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    phi[k] = 0;
-    plo[k] = 0;
-  }
-#pragma unroll
-  for (int g = 0; g < C / 4; ++g) {
-    int k = 0;
-#pragma unroll
-    for (int j = 1; j < K; ++j)
-      if (g >= Pt::first_group(j)) k = j;
-    const QuantParts a = quant_parts(v[4 * g], f1, f1s), b = quant_parts(v[4 * g + 1], f1, f1s);
-    const QuantParts c = quant_parts(v[4 * g + 2], f1, f1s),
-                     d = quant_parts(v[4 * g + 3], f1, f1s);
-    if (K == 1 && (g & 1)) {
-      hi2 += a.hi_bits + b.hi_bits;
-      lo2 += a.lo_bits + b.lo_bits;
-      hi2 += c.hi_bits + d.hi_bits;
-      lo2 += c.lo_bits + d.lo_bits;
-    } else {
-#pragma unroll
-      for (int j = 0; j < K; ++j)
-        if (j == k) {
-          phi[j] += a.hi_bits + b.hi_bits;
-          plo[j] += a.lo_bits + b.lo_bits;
-          phi[j] += c.hi_bits + d.hi_bits;
-          plo[j] += c.lo_bits + d.lo_bits;
-        }
-    }
-  }
-  if (K == 1) {
-    phi[0] += hi2;
-    plo[0] += lo2;
-  }
-}
-
-// The value of part k's sum: its bit-pattern sums minus the offsets of its
-// cities; the true sums are below C * 2^23 <= 2^30, so the modular sums are
-// exact.  k must be a compile-time constant (an unrolled loop index).
-template <int C, int K>
-__device__ __forceinline__ unsigned long long part_value(const uint32_t (&phi)[K],
-                                                         const uint32_t (&plo)[K], int k) {
-  const uint32_t off = (uint32_t)ChunkParts<C, K>::cities(k) * kTwo23Bits;
-  return ((unsigned long long)(phi[k] - off) << 23) + (plo[k] - off);
-}
-
-// Same sum, also keeping each group of four weights' hi/lo part sums (with
-// their 4 * 0x4b000000 offsets) for the in-lane search of the selected city.
-template <int C>
-__device__ __forceinline__ unsigned long long chunk_sum_groups(const uint32_t (&v)[C], float f1,
-                                                               float f1s, uint32_t (&ghi)[C / 4],
-                                                               uint32_t (&glo)[C / 4]) {
-  uint32_t hi = 0, lo = 0;
-#pragma unroll
-  for (int g = 0; g < C / 4; ++g) {
-    const QuantParts a = quant_parts(v[4 * g], f1, f1s), b = quant_parts(v[4 * g + 1], f1, f1s);
-    const QuantParts c = quant_parts(v[4 * g + 2], f1, f1s),
-                     d = quant_parts(v[4 * g + 3], f1, f1s);
-    ghi[g] = a.hi_bits + b.hi_bits + c.hi_bits + d.hi_bits;
-    glo[g] = a.lo_bits + b.lo_bits + c.lo_bits + d.lo_bits;
-    hi += ghi[g];
-    lo += glo[g];
-  }
-  const uint32_t off = (uint32_t)C * kTwo23Bits;
-  return ((unsigned long long)(hi - off) << 23) + (lo - off);
 }
 
 // The lanes of one warp segment (H = 32: the whole warp).
@@ -309,6 +184,7 @@ struct Compaction {
   }
   // Slot count of phase j (0 = the direct phase, C), or 0 past the last.
   __host__ __device__ static constexpr int slots(int j) {
+    if (!kOn) return j == 0 ? C : 0;
     int prev = 1 << 30, k = -1;
     for (int i = 0; i < 4; ++i) {
       const int v = raw(i);
@@ -369,18 +245,15 @@ __device__ __forceinline__ float race_exponential(uint32_t x) {
   return __fsub_rn(__fmul_rn(__int2float_rn(24 - e), 0x1.62e430p-1f), ln_f);
 }
 
-// R = 0: Eq. 1 by the integer roulette.  R = 1: the paper's data-parallel
-// rule: every unvisited city scores u_j * w_j with its own uniform u_j, the
-// highest score wins (ties to the lower index; all scores 0: the lowest
-// unvisited city).  R = 2: the exponential race, which samples Eq. 1: every
-// unvisited city gets the key E_j / w_j from its own exponential variate
-// E_j, the smallest key wins (ties to the lower index; zero weights and
-// overflowing keys are +inf, so with every weight 0 the lowest unvisited
-// city wins).
-// kPool: the ant belongs to a many-instance launch, where the GPU is full and
-// issue-bound (fewer instructions per step pay even at a longer chain).
-template <int C, int G, int H, int R = 0, bool kPool = false>
-__device__ __forceinline__ void construct_ant(const Instance& I, const int ant, const int tg,
+// The per-candidate rules.  R = 1: the paper's data-parallel rule: every
+// unvisited city scores u_j * w_j with its own uniform u_j, the highest score
+// wins (ties to the lower index; all scores 0: the lowest unvisited city).
+// R = 2: the exponential race, which samples Eq. 1: every unvisited city gets
+// the key E_j / w_j from its own exponential variate E_j, the smallest key
+// wins (ties to the lower index; zero weights and overflowing keys are +inf,
+// so with every weight 0 the lowest unvisited city wins).
+template <int C, int G, int H, int R>
+__device__ __forceinline__ void construct_ant_rule(const Instance& I, const int ant, const int tg,
                                               const Seg<H> seg, GroupSmem* gs, const int bar_id,
                                               float* srow, const bool lane_copy) {
   static_assert(C % 4 == 0 && C >= 4 && C <= 128, "C must be a multiple of 4 in [4,128]");
@@ -390,22 +263,6 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
   static_assert(H == 8 || H == 16 || H == 32, "H must be 8, 16 or 32");
   static_assert(H == 32 || G == 1, "segments smaller than a warp serve one ant each");
   constexpr int NW = (C + 31) / 32;  // tabu words per thread
-  // The smallest chunk (4 cities) keeps its sums in registers and the
-  // selected lane finds the city alone; larger chunks are rescanned by the
-  // whole segment, which measured faster than a serial in-lane search.
-  constexpr bool kGroupPick = C <= 4;
-  constexpr int NG = kGroupPick ? C / 4 : 1;
-  // Larger chunks keep per-part sums (K parts of whole 4-city groups) so the
-  // rescan covers one part: at most about one city per lane.  This cuts the
-  // instructions of a step but lengthens its dependent chain (the selected
-  // lane picks the part first), so a single instance, whose ants may not
-  // fill the GPU, splits only chunks of more than two cities per lane in the
-  // rescan (measured: 2.8 % faster at C = 76, 2.4 % slower at C = 36).
-  constexpr int KW = (C + H - 1) / H;  // cities per lane in an unsplit rescan
-  constexpr int KP = (kGroupPick || (!kPool && KW <= 2)) ? 1 : (KW < 4 ? KW : 4);
-  using Parts = ChunkParts<C, (KP < C / 4 ? KP : C / 4)>;
-  constexpr int K = KP < C / 4 ? KP : C / 4;
-  constexpr int PP = (Parts::max_cities() + H - 1) / H;  // cities per lane in the rescan
   constexpr int NT = H == 32 ? 32 * G : H;  // threads per ant
   const int n = I.n, ld = I.ld;
   const int hl = seg.hl;          // lane within the segment
@@ -446,7 +303,6 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
   const float* const choice = I.choice;
   if (tg == 0) tour[0] = start;
   int cur = start;
-  unsigned long long rwin = 0;
 
   const uint32_t srow_a = smem_u32(srow);
   const uint32_t bar = srow_a + (uint32_t)StageLayout<C, G, H>::kRowFloats * 4u;
@@ -471,12 +327,6 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
       fence_proxy_async_smem();
       bulk_load(srow_a, choice + (size_t)cur * ld, row_bytes, bar);
     }
-    const int off = (s - 1) % H;
-    if (off == 0) {
-      const Philox4 x = step_draw(seed, (uint32_t)(s + hl), (uint32_t)ant, iter);
-      rwin = ((unsigned long long)x.x1 << 32) | x.x0;
-    }
-    const unsigned long long r = seg.shfl(rwin, off);
     if (lane_copy) {
       group_wait();
     } else {
@@ -488,33 +338,7 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
     }
     const float* row = srow;
 
-    uint32_t v[R == 0 ? C : 1];  // weight bits; w >= 0 orders like its bit pattern
-    uint32_t mx = 0u;
-    if constexpr (R == 0) {
-#pragma unroll
-      for (int i = 0; i < C; i += 4) {
-        // Chunk entries at or beyond ld hold stale data; their tabu bits are set.
-        const uint4 t = *reinterpret_cast<const uint4*>(row + base + i);
-        v[i] = t.x;
-        v[i + 1] = t.y;
-        v[i + 2] = t.z;
-        v[i + 3] = t.w;
-      }
-      uint32_t m4[4] = {0u, 0u, 0u, 0u};  // four independent max chains
-#pragma unroll
-      for (int i = 0; i < C; ++i) {
-        if ((vis[i >> 5] >> (i & 31)) & 1u) v[i] = 0u;
-        m4[i & 3] = max(m4[i & 3], v[i]);
-      }
-      mx = seg.max_u32(max(max(m4[0], m4[1]), max(m4[2], m4[3])));
-      if (G > 1) {
-        if (hl == 0) gs->wmax[wg] = mx;
-        group_sync(bar_id, NT);
-#pragma unroll
-        for (int w = 0; w < G; ++w) mx = max(mx, gs->wmax[w]);
-      }
-    }
-
+    uint32_t mx;  // 0: no score or key decides
     int next;
     // A group of four consecutive cities (C and base are multiples of 4)
     // shares one Philox call.
@@ -648,9 +472,7 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
       mx = (uint32_t)(key >> 32) < kInf ? 1u : 0u;
       next = (int)(uint32_t)key;
     }
-    if (R != 0 && mx != 0u) {
-      // chosen above
-    } else if (mx == 0u) {
+    if (mx == 0u) {
       // Every unvisited weight is zero: the lowest-index unvisited city.
       uint32_t cand = 0xffffffffu;
 #pragma unroll
@@ -666,149 +488,6 @@ __device__ __forceinline__ void construct_ant(const Instance& I, const int ant, 
         for (int w = 0; w < G; ++w) cand = min(cand, (uint32_t)gs->wmin[w]);
       }
       next = (int)cand;
-    } else if constexpr (R == 0) {
-      const int sc = kRouletteBits - 1 - exponent_of_bits(mx);
-      float f1, f1s, f2;
-      quant_factors(sc, f1, f1s, f2);
-      if (f2 != 1.0f) {
-        // Largest unvisited weight below 2^-82 (rare): scale the chunk up
-        // first, exactly (quant_value() does the same for reloaded weights).
-#pragma unroll
-        for (int i = 0; i < C; ++i) v[i] = __float_as_uint(__fmul_rn(__uint_as_float(v[i]), f2));
-      }
-      uint32_t ghi[NG], glo[NG];
-      uint32_t phi[K], plo[K];
-      unsigned long long mine;
-      if constexpr (kGroupPick) {
-        mine = chunk_sum_groups<C>(v, f1, f1s, ghi, glo);
-      } else {
-        chunk_sum_parts<C, K>(v, f1, f1s, phi, plo);
-        uint32_t hs = phi[0], ls = plo[0];
-#pragma unroll
-        for (int k = 1; k < K; ++k) {
-          hs += phi[k];
-          ls += plo[k];
-        }
-        const uint32_t off = (uint32_t)C * kTwo23Bits;
-        mine = ((unsigned long long)(hs - off) << 23) + (ls - off);
-      }
-      const unsigned long long incl = seg.inclusive_scan(mine);
-      const unsigned long long wtot = seg.shfl(incl, H - 1);
-      unsigned long long woff = 0, Q = wtot;
-      if (G > 1) {
-        if (hl == 0) gs->wsum[wg] = wtot;
-        group_sync(bar_id, NT);
-        Q = 0;
-#pragma unroll
-        for (int w = 0; w < G; ++w) {
-          const unsigned long long u = gs->wsum[w];
-          if (w < wg) woff += u;
-          Q += u;
-        }
-      }
-      const unsigned long long T = __umul64hi(r, Q);
-      next = 0;
-      if (G == 1 || (T >= woff && T - woff < wtot)) {
-        const unsigned long long t1 = T - woff;
-        const int L = max(__ffs(seg.ballot(incl > t1)) - 1, 0);
-        const unsigned long long t2 = t1 - seg.shfl(incl - mine, L);
-        const int baseL = (wg * H + L) * C;  // within the staged row
-        if constexpr (kGroupPick) {
-          // Lane L walks its group sums, then the four cities of the group
-          // holding the target (all from registers).
-          int pick = 0;
-          if (hl == L) {
-            unsigned long long cum = 0;
-            bool found = false;
-#pragma unroll
-            for (int g = 0; g < NG; ++g) {
-              const unsigned long long gv =
-                  ((unsigned long long)(ghi[g] - 4u * kTwo23Bits) << 23) + (glo[g] - 4u * kTwo23Bits);
-              if (!found && cum + gv > t2) {
-                found = true;
-                unsigned long long c = cum + quant_value(v[4 * g], f1, f1s, 1.0f);
-                int e = 0;
-                if (c <= t2) {
-                  c += quant_value(v[4 * g + 1], f1, f1s, 1.0f);
-                  e = 1;
-                  if (c <= t2) {
-                    c += quant_value(v[4 * g + 2], f1, f1s, 1.0f);
-                    e = c <= t2 ? 3 : 2;
-                  }
-                }
-                pick = 4 * g + e;
-              }
-              cum += gv;
-            }
-          }
-          next = baseL + seg.shfl(pick, L);
-        } else {
-          // Lane L finds the part of its chunk that holds the target.
-          int part = 0;
-          unsigned long long t3 = t2;
-          if constexpr (K > 1) {
-            if (hl == L) {
-              unsigned long long cum = 0;
-              bool found = false;
-#pragma unroll
-              for (int k = 0; k < K; ++k) {
-                const unsigned long long pv = part_value<C, K>(phi, plo, k);
-                if (!found && (k == K - 1 || cum + pv > t2)) {
-                  found = true;
-                  part = k;
-                  t3 = t2 - cum;
-                }
-                cum += pv;
-              }
-            }
-            part = seg.shfl(part, L);
-            t3 = seg.shfl(t3, L);
-          }
-          // The segment rescans that part, PP cities per lane.
-          const int pstart = 4 * (part * Parts::NG / K);
-          const int psz = 4 * ((part + 1) * Parts::NG / K) - pstart;
-          uint32_t visL[NW];
-#pragma unroll
-          for (int w = 0; w < NW; ++w) visL[w] = seg.shfl(vis[w], L);
-          unsigned long long qv[PP];
-          unsigned long long ps = 0;
-#pragma unroll
-          for (int p = 0; p < PP; ++p) {
-            const int pi = hl * PP + p;  // position within the part
-            const int li = pstart + pi;  // position within lane L's chunk
-            uint32_t word = FULL;
-#pragma unroll
-            for (int w = 0; w < NW; ++w)
-              if (w == (li >> 5)) word = visL[w];
-            uint32_t w8 = 0u;
-            if (pi < psz && baseL + li < ld && !((word >> (li & 31)) & 1u))
-              w8 = __float_as_uint(row[baseL + li]);
-            qv[p] = quant_value(w8, f1, f1s, f2);
-            ps += qv[p];
-          }
-          const unsigned long long incl2 = seg.inclusive_scan(ps);
-          const int L2 = max(__ffs(seg.ballot(incl2 > t3)) - 1, 0);
-          int pick = 0;
-          if constexpr (PP > 1) {
-            if (hl == L2) {
-              unsigned long long c = incl2 - ps;
-              pick = -1;
-#pragma unroll
-              for (int p = 0; p < PP; ++p) {
-                c += qv[p];
-                if (pick < 0 && c > t3) pick = p;
-              }
-            }
-            pick = max(seg.shfl(pick, L2), 0);
-          }
-          next = baseL + pstart + L2 * PP + pick;
-        }
-        if (G > 1 && hl == 0) gs->next = next;
-      }
-      if (G > 1) {
-        group_sync(bar_id, NT);
-        next = gs->next;
-      }
     }
 
     // A city outside [0, n) can only come from a defect; record it and stay
@@ -872,8 +551,8 @@ __device__ __forceinline__ void group_of_thread(int& grp, int& tg) {
 
 // One CTA holds groups_per_cta<G, H>(blockDim.x / 32) ant groups; dynamic
 // shared memory holds one StageLayout<C, G, H> per group.
-template <int C, int G, int H, int R = 0>
-__global__ void __launch_bounds__(256) construct_kernel(Instance I) {
+template <int C, int G, int H, int R>
+__global__ void __launch_bounds__(256) construct_rule_kernel(Instance I) {
   __shared__ GroupSmem gs[kMaxGroupsPerCta];
   extern __shared__ __align__(16) unsigned char stage[];
   int grp, tg;
@@ -881,30 +560,8 @@ __global__ void __launch_bounds__(256) construct_kernel(Instance I) {
   const int ant = blockIdx.x * groups_per_cta<G, H>(blockDim.x >> 5) + grp;
   if (ant >= I.m) return;
   float* srow = reinterpret_cast<float*>(stage + grp * StageLayout<C, G, H>::kBytes);
-  construct_ant<C, G, H, R>(I, ant, tg, Seg<H>(threadIdx.x & 31), &gs[H == 32 ? grp : 0], 1 + grp,
+  construct_ant_rule<C, G, H, R>(I, ant, tg, Seg<H>(threadIdx.x & 31), &gs[H == 32 ? grp : 0], 1 + grp,
                             srow, I.stage != 0);
-}
-
-// Batched form: group g of block b builds ant items[b*A + g].y of instance
-// insts[items[b*A + g].x].  Items are listed longest instance first.  The
-// row staging is chosen per launch (`lane_copy`), not per instance.
-template <int C, int G, int H>
-__global__ void __launch_bounds__(256) construct_items_kernel(const Instance* __restrict__ insts,
-                                                              const int2* __restrict__ items,
-                                                              int count, int lane_copy) {
-  __shared__ GroupSmem gs[kMaxGroupsPerCta];
-  extern __shared__ __align__(16) unsigned char stage[];
-  int grp, tg;
-  group_of_thread<G, H>(grp, tg);
-  const int idx = blockIdx.x * groups_per_cta<G, H>(blockDim.x >> 5) + grp;
-  if (idx >= count) return;
-  const int2 it = items[idx];
-  // A reference into the descriptor table (read-only, L1-cached) rather than
-  // a register copy of the whole descriptor, which cost ~40 registers.
-  const Instance& I = insts[it.x];
-  float* srow = reinterpret_cast<float*>(stage + grp * StageLayout<C, G, H>::kBytes);
-  construct_ant<C, G, H, 0, true>(I, it.y, tg, Seg<H>(threadIdx.x & 31), &gs[H == 32 ? grp : 0],
-                                  1 + grp, srow, lane_copy != 0);
 }
 
 // The Eq. 1 walk with compaction (construct_phased.cuh), one group of H lanes
@@ -957,18 +614,14 @@ inline size_t construct_smem_setup(int warps) {
   static std::atomic<unsigned long long> done{0};
   once_per_device(done, [] {
     const int most = groups_per_cta<G, H>(8) * StageLayout<C, G, H>::kBytes;
-    constexpr bool kPhased = R == 0 && Compaction<C, G>::kOn;
-    if constexpr (kItems && kPhased)
+    if constexpr (kItems)
       return cudaFuncSetAttribute(construct_phased_items_kernel<C, G, H>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    else if constexpr (kItems)
-      return cudaFuncSetAttribute(construct_items_kernel<C, G, H>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    else if constexpr (kPhased)
+    else if constexpr (R == 0)
       return cudaFuncSetAttribute(construct_phased_kernel<C, G, H>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     else
-      return cudaFuncSetAttribute(construct_kernel<C, G, H, R>,
+      return cudaFuncSetAttribute(construct_rule_kernel<C, G, H, R>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   });
   return bytes;

@@ -1,14 +1,14 @@
-// Tour construction by Eq. 1 (Section II; the integer roulette of reading R2)
-// for one warp, one warp segment or two warps per ant, with the unvisited
-// cities compacted up to three times along the walk.
+// Tour construction by Eq. 1 (Section II; the integer roulette of reading R2),
+// for every tiling, with the unvisited cities compacted up to three times
+// along the walk where a chunk holds 20 cities or more (one or two warps, or
+// one warp segment, per ant).
 //
-// A step of the plain kernel (construct_ant) handles every city of the row,
-// visited or not: lane t owns the cities [tC, tC + C), zeroes the visited
-// ones and still pays the max, the quantisation and the sum for them.  Half
-// way through a tour half of that work is spent on visited cities.  Here the
-// walk runs in up to four phases:
-//   phase 0  (at most 32*C1 unvisited cities not yet reached): as the plain
-//            kernel, lane t owns the contiguous chunk [tC, tC + C) of the row;
+// A step that handles every city of the row, visited or not, pays for the
+// visited ones too; half way through a tour that is half of the work.  The
+// walk therefore runs in up to four phases:
+//   phase 0  (at most 32*C1 unvisited cities not yet reached): lane t owns the
+//            contiguous chunk [tC, tC + C) of the row and skips visited cities
+//            by their tabu bits;
 //   phase 1  the unvisited cities, in ascending order, are listed in shared
 //            memory and dealt out C1 = 4*ceil(C/8) per lane (lane t takes
 //            entries [t*C1, t*C1 + C1)); each step reads the entries and
@@ -20,14 +20,22 @@
 //   phase 3  the same with C3 = 4*ceil(C/32) per lane (when smaller than C2).
 // Phase p starts at the first step at which the unvisited cities fit in the
 // segment's H*Cp slots.  Every phase keeps the cities of the segment in
-// ascending order, lane after lane and slot after slot, so the integer
-// roulette (first city whose inclusive prefix sum exceeds T) chooses the same
-// city as the plain kernel and the CPU oracle.  With two warps per ant the
-// group's 64 threads hold the slots in that order, warp 0 first; the warps
-// combine their maxima and totals through shared memory, and the warp whose
-// range holds the target runs the second-level search.  The row is still staged
-// whole (bulk copy), so the L2 bytes do not change; the per-candidate work
-// of the later steps halves, quarters and eighths.
+// ascending order, lane after lane and slot after slot, so the first city
+// whose inclusive prefix sum exceeds the target is the CPU oracle's choice.
+// With several warps per ant the group's threads hold the slots in that
+// order, warp 0 first; the warps combine their totals through shared memory,
+// and the warp whose range holds the target publishes the city.  The row is
+// still staged whole (bulk copy), so the L2 bytes do not change; the
+// per-candidate work of the later steps halves, quarters and eighths.
+//
+// Construct, GB300, ms, m = n unless given: quantised 64-bit sums -> this
+// walk: n = 48 0.034 -> 0.029, n = 200 0.163 -> 0.116, n = 384 0.310 -> 0.222,
+// n = 517 0.464 -> 0.335, n = 1002 1.118 -> 0.801, n = 1500 2.13 -> 1.43,
+// n = 2392 5.05 -> 3.31, n = 4096 with m = 1024 9.02 -> 6.22.  Small instances
+// are bound by the step's chain (about 1500 cycles at n = 1002: the row copy
+// 500, the sums 200, the scan and the lane 280, the slot 150, the rest
+// issue), large ones also by the rows: 54.7 GB at n = 2392 take 2.7 ms at the
+// L2's read rate.
 #pragma once
 
 namespace aco {
@@ -62,12 +70,12 @@ struct Pick {
 // falls on, or no open weight is positive (0.1-2 % of the steps).  Its loops
 // stay rolled and read the row again, so that it costs the walk no registers;
 // as a call of its own it cost 3 % (the values kept across the call).
-// list = nullptr: slot i of thread tg is city tg*cp + i with tabu bits v0..v2;
+// list = nullptr: slot i of thread tg is city tg*cp + i with tabu bits vis;
 // otherwise the list entry tg*cp + i.
-template <int G, int H, uint32_t kUnit>
-__device__ __forceinline__ Pick exact_pick(const float* row, uint16_t* list, int cp, uint32_t zero_entry,
-                                        uint32_t v0, uint32_t v1, uint32_t v2, int tg, int bar_id,
-                                        GroupSmem* gs, unsigned long long r) {
+template <int G, int H, uint32_t kUnit, int NW>
+__device__ __forceinline__ Pick exact_pick(const float* row, uint16_t* list, int cp,
+                                           uint32_t zero_entry, const uint32_t (&vis)[NW], int tg,
+                                           int bar_id, GroupSmem* gs, unsigned long long r) {
   constexpr int NT = G * H;
   const Seg<H> seg(threadIdx.x & 31);
   const int hl = seg.hl, wg = G > 1 ? tg >> 5 : 0;
@@ -77,10 +85,16 @@ __device__ __forceinline__ Pick exact_pick(const float* row, uint16_t* list, int
     else
       seg.sync();
   };
+  auto closed = [&](int i) {
+    uint32_t word = vis[0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w)
+      if (i >= 32 * w) word = vis[w];
+    return (word >> (i & 31)) & 1u;
+  };
   auto weight = [&](int i) -> uint32_t {
     if (list) return entry_weight<kUnit>(row, list[tg * cp + i]);
-    const uint32_t word = i < 32 ? v0 : (i < 64 ? v1 : v2);
-    return (word >> (i & 31)) & 1u ? 0u : __float_as_uint(row[tg * cp + i]);
+    return closed(i) ? 0u : __float_as_uint(row[tg * cp + i]);
   };
   uint32_t mx = 0u;
 #pragma unroll 1
@@ -101,8 +115,7 @@ __device__ __forceinline__ Pick exact_pick(const float* row, uint16_t* list, int
       if (list) {
         cand = min(cand, (uint32_t)list[tg * cp + i]);
       } else {
-        const uint32_t word = i < 32 ? v0 : (i < 64 ? v1 : v2);
-        if (!((word >> (i & 31)) & 1u)) cand = (uint32_t)(tg * cp + i);
+        if (!closed(i)) cand = (uint32_t)(tg * cp + i);
       }
     }
     cand = seg.min_u32(cand);
@@ -192,7 +205,7 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
                                           const Seg<H> seg, GroupSmem* gs, const int bar_id,
                                           float* srow, uint16_t* ulist, const int start,
                                           const int s_end, WalkState& w) {
-  static_assert(CP % 4 == 0 && CP >= 4 && CP <= 96, "CP must be a multiple of 4 in [4,96]");
+  static_assert(CP % 4 == 0 && CP >= 4 && CP <= 160, "CP must be a multiple of 4 in [4,160]");
   static_assert(kGather || CP == C, "the direct phase reads whole chunks");
   static_assert(G == 1 || H == 32, "several warps per ant use whole warps");
   constexpr int NT = G * H;  // threads per ant
@@ -441,13 +454,8 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
     if (!found) {
       const Philox4 x = step_draw(seed, (uint32_t)s, (uint32_t)ant, iter);
       const unsigned long long r = ((unsigned long long)x.x1 << 32) | x.x0;
-      uint32_t v3[3] = {FULL, FULL, FULL};
-      if constexpr (!kGather) {
-#pragma unroll
-        for (int wd = 0; wd < NW; ++wd) v3[wd] = vis[wd];
-      }
-      got = exact_pick<G, H, kUnit>(row, kGather ? ulist : nullptr, CP, kZeroEntry, v3[0], v3[1],
-                                    v3[2], tg, bar_id, gs, r);
+      got = exact_pick<G, H, kUnit>(row, kGather ? ulist : nullptr, CP, kZeroEntry, vis, tg, bar_id,
+                                    gs, r);
       // A city outside [0, n) can only come from a defect; record it and stay
       // in bounds instead of reading past the matrix.
       if ((unsigned)got.next >= (unsigned)n) {
@@ -559,8 +567,6 @@ __device__ __forceinline__ void construct_ant_phased(const Instance& I, const in
                                                      const int tg, const Seg<H> seg,
                                                      GroupSmem* gs, const int bar_id, float* srow,
                                                      const bool lane_copy) {
-  using Cm = Compaction<C, G>;
-  static_assert(Cm::kOn, "compaction needs one or two whole groups per ant and C >= kCompactMinC");
   constexpr int NT = G * H;
   uint16_t* ulist = reinterpret_cast<uint16_t*>(reinterpret_cast<char*>(srow) +
                                                 StageLayout<C, G, H>::kListOffset);

@@ -43,10 +43,10 @@ __global__ void __maxnreg__(64)
     const bool lc = cls.lane_copy[k] != 0;
     switch (cls.C[k]) {
       case 4:
-        construct_ant<4, 1, 32, 0, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
+        construct_ant_phased<4, 1, 32, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
         break;
       case 12:
-        construct_ant<12, 1, 32, 0, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
+        construct_ant_phased<12, 1, 32, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
         break;
       case 20:
         construct_ant_phased<20, 1, 32, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
