@@ -323,14 +323,10 @@ __device__ __forceinline__ void construct_ant_rule(const Instance& I, const int 
       const float4* src = reinterpret_cast<const float4*>(choice + (size_t)cur * ld);
       float4* dst = reinterpret_cast<float4*>(srow);
       for (int i = tg; i < (ld >> 2); i += NT) dst[i] = src[i];
-    } else if (tg == 0) {
-      fence_proxy_async_smem();
-      bulk_load(srow_a, choice + (size_t)cur * ld, row_bytes, bar);
-    }
-    if (lane_copy) {
       group_wait();
     } else {
-      if (waits_ok && !mbar_wait_bounded(bar, phase)) {
+      bulk_load_if(tg == 0, srow_a, choice + (size_t)cur * ld, row_bytes, bar);
+      if (!mbar_try_wait(bar, phase) && waits_ok && !mbar_wait_bounded(bar, phase)) {
         waits_ok = false;  // stale data from here on; the status word says so
         if (tg == 0) atomicOr(&I.st->status, kStatusTimeout);
       }
@@ -572,13 +568,21 @@ __global__ void __launch_bounds__(256) construct_rule_kernel(Instance I) {
 // against 1.98 at 72; a step of 256 instances 14.3 ms against 14.5; 48 and 56
 // are 1-2 % slower everywhere); above, the rows limit the ants and 128 costs
 // nothing (n = 2392 3.30 ms; 96: 3.32, 72: 3.34).
-template <int C>
+// Two warps per ant (n > 2432) would hold 2 x 13 warps at C = 52 and 2 x 11 at
+// C = 60 by their rows: ceilings that let them all reside (n = 3100 11.6 ms at
+// 128, 9.73 at 72).
+template <int C, int G>
 struct PhasedRegs {
-  static constexpr int v = C <= 36 ? 64 : 128;
+  static constexpr int v = C <= 36               ? 64
+                           : G == 1              ? 128
+                           : C <= 44             ? 64
+                           : C <= 52             ? 72
+                           : C <= 60             ? 80
+                                                 : 96;
 };
 
 template <int C, int G, int H>
-__global__ void __maxnreg__((PhasedRegs<C>::v)) construct_phased_kernel(Instance I) {
+__global__ void __maxnreg__((PhasedRegs<C, G>::v)) construct_phased_kernel(Instance I) {
   __shared__ GroupSmem gs[kMaxGroupsPerCta];
   extern __shared__ __align__(16) unsigned char stage[];
   int grp, tg;
@@ -591,7 +595,7 @@ __global__ void __maxnreg__((PhasedRegs<C>::v)) construct_phased_kernel(Instance
 }
 
 template <int C, int G, int H>
-__global__ void __maxnreg__((PhasedRegs<C>::v))
+__global__ void __maxnreg__((PhasedRegs<C, G>::v))
     construct_phased_items_kernel(const Instance* __restrict__ insts,
                                   const int2* __restrict__ items, int count, int lane_copy) {
   __shared__ GroupSmem gs[kMaxGroupsPerCta];
