@@ -105,7 +105,11 @@ extern "C" {
                                   completing on an mbarrier; 1 coalesced
                                   16-byte loads by the ant's threads.  Default:
                                   1 for n <= 64, else 0 (the faster measured
-                                  on GB300).  Results are identical.          */
+                                  on GB300).  Results are identical.  (With
+                                  the default tiling, Eq. 1 instances of n <=
+                                  240 bring the whole choice_info matrix into
+                                  shared memory once per construction and
+                                  stage no rows.)                             */
 
 #define ACO_SELECT_EQ1 0       /* Eq. 1 (random proportional rule), exact      */
 #define ACO_SELECT_DATA_PARALLEL 1 /* the paper's data-parallel kernel (Section

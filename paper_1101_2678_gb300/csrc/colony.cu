@@ -217,11 +217,15 @@ static void drop_graph(aco_colony* h) {
 static int enqueue_construct(aco_colony* h) {
   const ConstructTiling t = tiling_of(h);
   if (!tiling_ok(t, h->I.rule)) return fail(ACO_EINVAL, "no construction tiling for n=%d", h->I.n);
+  // the default tiling only: options that name a tiling get that one
+  const bool small = h->I.rule == 0 && !h->warps_per_ant && !h->lanes_per_ant &&
+                     !h->ants_per_cta && construct_small_fits(h->I.n);
   cudaError_t e;
   if (h->profile && (e = record_event(h, h->ev[0], h->stream)) != cudaSuccess)
     return cuda_fail(e, "event");
   e = h->I.variant == kVariantAcs ? launch_acs_construct(h->I, h->stream)
       : h->I.nn > 0               ? launch_construct_nn(h->I, h->stream)
+      : small                     ? launch_construct_small(h->I, h->sms, h->stream)
                                   : launch_construct(h->I, t, h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "construct");
   if (h->profile && (e = record_event(h, h->ev[1], h->stream)) != cudaSuccess)

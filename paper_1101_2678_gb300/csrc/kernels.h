@@ -81,6 +81,10 @@ bool construct_supported(int C, int G, int H);
 // The paper's data-parallel selection rule (Instance::rule == 1); H = 32, G = 1 or 2.
 cudaError_t launch_construct_rule1(const Instance& I, ConstructTiling t, cudaStream_t st);
 cudaError_t launch_construct_rule2(const Instance& I, ConstructTiling t, cudaStream_t st);
+// Eq. 1 with the whole choice_info matrix in shared memory (construct_small.cu),
+// for the default tiling where construct_small_fits().
+bool construct_small_fits(int n);
+cudaError_t launch_construct_small(const Instance& I, int sms, cudaStream_t st);
 cudaError_t launch_construct_items(const Instance* insts, const int2* items, int count,
                                    ConstructTiling t, cudaStream_t st);
 // One persistent launch over the items of several classes (whole warps per
