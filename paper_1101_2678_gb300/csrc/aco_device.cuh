@@ -24,6 +24,37 @@ inline cudaError_t once_per_device(std::atomic<unsigned long long>& done, F set)
   return e;
 }
 
+// Host: launch `kernel` so that its CTAs may start before the stream's previous
+// kernel has ended (programmatic dependent launch): the kernel calls
+// grid_wait() before it touches anything that kernel wrote or read, and the
+// previous kernel calls grid_release() once its successor may come in.
+template <class... P, class... A>
+inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// Wait until the previous kernel has completed and its writes are visible
+// (nothing to wait for after an ordinary launch).
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Let the next kernel's CTAs in once every CTA of this one has said so or ended.
+__device__ __forceinline__ void grid_release() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Per-instance iteration state, resident on the device.
 struct IterState {
   unsigned long long iteration;  // completed pheromone updates (Philox counter word 2)
@@ -157,6 +188,15 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 // 2^e as a double, for -1022 <= e <= 1023.
 __device__ __forceinline__ double pow2d(int e) {
   return __longlong_as_double((long long)(e + 1023) << 52);
+}
+
+// floor(d * 2^shift) for a float d >= 0 by its significand (the FP64 units are
+// few: a conversion there costs as much as a warp's whole integer shift).
+__device__ __forceinline__ unsigned long long fixed_of(float d, int shift) {
+  const uint32_t b = __float_as_uint(d);
+  const unsigned long long sig = b >= 0x00800000u ? (b & 0x007fffffu) | 0x00800000u : b;
+  const int e = (b >= 0x00800000u ? (int)(b >> 23) : 1) - 150 + shift;  // d = sig 2^(e - shift)
+  return e >= 0 ? sig << e : (e > -64 ? sig >> -e : 0ull);
 }
 
 __device__ __forceinline__ unsigned long long shfl_u64(unsigned long long v, int src) {
