@@ -59,10 +59,45 @@ __global__ void nn_choice_kernel(Instance I) {
   }
 }
 
+// The unvisited city of the row's largest choice_info, ties to the lower index.
+// The bits of non-negative floats order like their values; an unvisited city's
+// key is bits + 1, a visited one's 0.  Each lane keeps the first of its largest
+// keys over its cities in ascending order.
+__device__ __forceinline__ int nn_dense_choice(const float* row, int n, const uint32_t* bits,
+                                               int lane) {
+  uint32_t bkey = 0u, bj = 0u;
+#pragma unroll 4
+  for (int j0 = 4 * lane; j0 < n; j0 += 128) {
+    // (rows are padded to a multiple of 4 with zeros)
+    const uint4 w4 = *reinterpret_cast<const uint4*>(row + j0);
+    const uint32_t fr = ~bits[j0 >> 5] >> (j0 & 31);
+    const uint32_t wv[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t key = ((fr >> e) & 1u) && j0 + e < n ? wv[e] + 1u : 0u;
+      if (key > bkey) {
+        bkey = key;
+        bj = (uint32_t)(j0 + e);
+      }
+    }
+  }
+  const uint32_t best = __reduce_max_sync(FULL, bkey);
+  return (int)__reduce_min_sync(FULL, bkey == best ? bj : 0xffffffffu);
+}
+
 // One warp per ant; lane l holds list entry l of the current city.  The
-// tabu list is a bitmap of n bits in shared memory (one per warp).
+// tabu list is a bitmap of n bits in shared memory (one per warp).  A step is
+// one chain: the list entry and its value, the tabu bit, the sums, the city.
+// The sums are single-precision prefix sums with an error bound, as in
+// eq1_phase() (construct_phased.cuh); where they cannot tell the city, the
+// integer roulette decides.  nn = 30, GB300, ms, quantised 64-bit sums -> this:
+// n = 1002 0.612 -> 0.468, n = 2392 1.89 -> 1.38 (a step 1200 cycles, a third of
+// them the loads).
 __device__ __forceinline__ void nn_construct_ant(const Instance& I, const int ant, const int lane,
                                                  uint32_t* bits) {
+  // roundings: the scan and the whole sum, the target, the differences, two to
+  // spare
+  constexpr float kEps = (float)(2 * 5 + 8) * 0x1p-24f;
   const int n = I.n, nn = I.nn, ld = I.ld, words = (n + 31) >> 5;
   const uint32_t iter = (uint32_t)I.st->iteration;
   const unsigned long long seed = I.seed;
@@ -76,61 +111,52 @@ __device__ __forceinline__ void nn_construct_ant(const Instance& I, const int an
     tour[0] = start;
   }
   __syncwarp();
+  const Seg<32> seg(lane);
   int cur = start;
-  unsigned long long rwin = 0;
+  float u = 0.0f;
   for (int s = 1; s < n; ++s) {
-    const int off = (s - 1) & 31;
-    if (off == 0) {
-      const Philox4 x = step_draw(seed, (uint32_t)(s + lane), (uint32_t)ant, iter);
-      rwin = ((unsigned long long)x.x1 << 32) | x.x0;
-    }
-    const unsigned long long r = shfl_u64(rwin, off);
     int j = 0;
-    uint32_t wb = 0u;
+    float w = 0.0f;
     bool unv = false;
     if (lane < nn) {
       j = I.nnlist[(size_t)cur * kNnStride + lane];
-      wb = __float_as_uint(I.nnchoice[(size_t)cur * kNnStride + lane]);
-      unv = !((bits[j >> 5] >> (j & 31)) & 1u);
+      w = I.nnchoice[(size_t)cur * kNnStride + lane];
     }
-    const uint32_t any = __ballot_sync(FULL, unv);
-    int next;
-    if (any) {
-      const uint32_t wm = unv ? wb : 0u;
-      const uint32_t mx = __reduce_max_sync(FULL, wm);
-      if (mx == 0u) {
-        next = __shfl_sync(FULL, j, __ffs(any) - 1);  // first unvisited entry
-      } else {
-        float f1, f1s, f2;
-        quant_factors(kRouletteBits - 1 - exponent_of_bits(mx), f1, f1s, f2);
-        const unsigned long long q = quant_value(wm, f1, f1s, f2);
-        unsigned long long incl = q;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned long long t = __shfl_up_sync(FULL, incl, o);
-          if (lane >= o) incl += t;
+    const int off = (s - 1) & 31;
+    if (off == 0) {
+      const Philox4 x = step_draw(seed, (uint32_t)(s + lane), (uint32_t)ant, iter);
+      u = __fmul_rn(__uint2float_rn(x.x1), 0x1p-32f);
+    }
+    const float us = __shfl_sync(FULL, u, off);
+    unv = lane < nn && !((bits[j >> 5] >> (j & 31)) & 1u);
+    if (!unv) w = 0.0f;
+    const float incl = seg.inclusive_scan_f(w);
+    const float S = __shfl_sync(FULL, incl, 31);
+    const float t = __fmul_rn(us, S);
+    const float err = S >= 0x1p-120f ? __fmul_rn(kEps, S) : __int_as_float(0x7f800000);
+    const uint32_t sure = __ballot_sync(
+        FULL, incl > __fadd_rn(t, err) && __fsub_rn(incl, w) < __fsub_rn(t, err));
+    int next = __shfl_sync(FULL, j, max(__ffs(sure) - 1, 0));
+    if (sure == 0u) {
+      const uint32_t any = __ballot_sync(FULL, unv);
+      if (any) {
+        const uint32_t mx = __reduce_max_sync(FULL, __float_as_uint(w));
+        if (mx == 0u) {
+          next = __shfl_sync(FULL, j, __ffs(any) - 1);  // first unvisited entry
+        } else {
+          const Philox4 x = step_draw(seed, (uint32_t)s, (uint32_t)ant, iter);
+          const unsigned long long r = ((unsigned long long)x.x1 << 32) | x.x0;
+          float f1, f1s, f2;
+          quant_factors(kRouletteBits - 1 - exponent_of_bits(mx), f1, f1s, f2);
+          const unsigned long long q =
+              seg.inclusive_scan(quant_value(__float_as_uint(w), f1, f1s, f2));
+          const unsigned long long T = __umul64hi(r, shfl_u64(q, 31));
+          next = __shfl_sync(FULL, j, max(__ffs(__ballot_sync(FULL, q > T)) - 1, 0));
         }
-        const unsigned long long T = __umul64hi(r, shfl_u64(incl, 31));
-        const int L = max(__ffs(__ballot_sync(FULL, incl > T)) - 1, 0);
-        next = __shfl_sync(FULL, j, L);
+      } else {
+        // every list entry is visited
+        next = nn_dense_choice(I.choice + (size_t)cur * ld, n, bits, lane);
       }
-    } else {
-      // Every list entry is visited: the heaviest unvisited city, ties to
-      // the lower index ((weight bits << 32) | ~j, maximised).
-      const float* row = I.choice + (size_t)cur * ld;
-      unsigned long long key = 0;
-      for (int jj = lane; jj < n; jj += 32) {
-        if ((bits[jj >> 5] >> (jj & 31)) & 1u) continue;
-        const unsigned long long k =
-            ((unsigned long long)__float_as_uint(row[jj]) << 32) | (0xffffffffu - (uint32_t)jj);
-        key = k > key ? k : key;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(FULL, key, o);
-        key = other > key ? other : key;
-      }
-      next = (int)(0xffffffffu - (uint32_t)key);
     }
     if ((unsigned)next >= (unsigned)n) {
       if (lane == 0) atomicOr(&I.st->status, kStatusBadTour);
