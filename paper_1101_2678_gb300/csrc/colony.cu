@@ -462,6 +462,7 @@ int aco_choice_info(aco_handle h, float* out) {
   if (e != cudaSuccess) return cuda_fail(e, "choice");
   if (out) {
     const int n = h->I.n;
+    touch_pages(out, (size_t)n * n * 4);
     e = cudaMemcpy2DAsync(out, (size_t)n * 4, h->I.choice, (size_t)h->I.ld * 4, (size_t)n * 4, n,
                           cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "copy choice");
@@ -479,6 +480,8 @@ int aco_construct_tours(aco_handle h, int32_t* tours, int64_t* lens) {
   h->constructed = true;
   cudaError_t e;
   const int n = h->I.n, m = h->I.m;
+  if (tours) touch_pages(tours, (size_t)m * (n + 1) * 4);
+  if (lens) touch_pages(lens, (size_t)m * 8);
   if (tours &&
       (e = cudaMemcpy2DAsync(tours, (size_t)(n + 1) * 4, h->I.tours, (size_t)h->I.ldt * 4,
                              (size_t)(n + 1) * 4, m, cudaMemcpyDeviceToHost, h->stream)) !=
@@ -559,6 +562,7 @@ int aco_best_tour(aco_handle h, int32_t* tour, int64_t* len) {
 int aco_get_pheromone(aco_handle h, float* tau) {
   if (!h || !tau) return fail(ACO_EINVAL, "NULL argument");
   const int n = h->I.n;
+  touch_pages(tau, (size_t)n * n * 4);
   cudaError_t e = cudaMemcpy2DAsync(tau, (size_t)n * 4, h->I.tau, (size_t)h->I.ld * 4,
                                     (size_t)n * 4, n, cudaMemcpyDeviceToHost, h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "copy tau");
@@ -568,6 +572,7 @@ int aco_get_pheromone(aco_handle h, float* tau) {
 int aco_get_heuristic(aco_handle h, float* heta) {
   if (!h || !heta) return fail(ACO_EINVAL, "NULL argument");
   const int n = h->I.n;
+  touch_pages(heta, (size_t)n * n * 4);
   cudaError_t e = cudaMemcpy2DAsync(heta, (size_t)n * 4, h->I.heta, (size_t)h->I.ld * 4,
                                     (size_t)n * 4, n, cudaMemcpyDeviceToHost, h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "copy heta");
@@ -639,6 +644,7 @@ int aco_save_state(aco_handle h, void* buf, uint64_t capacity, uint64_t* size) {
   if (!buf) return ACO_OK;
   if (capacity < *size) return fail(ACO_EINVAL, "buffer holds %llu bytes, %llu needed",
                                     (unsigned long long)capacity, (unsigned long long)*size);
+  touch_pages(buf, *size);
   CheckpointHeader hd = checkpoint_header(h->I);
   hd.constructed = h->constructed ? 1 : 0;
   hd.host_iteration = h->host_iteration;

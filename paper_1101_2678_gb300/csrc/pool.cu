@@ -992,6 +992,7 @@ int aco_pool_save_slot(aco_pool_handle p, int32_t slot, void* buf, uint64_t capa
   if (!buf) return ACO_OK;
   if (capacity < *size) return fail(ACO_EINVAL, "buffer holds %llu bytes, %llu needed",
                                     (unsigned long long)capacity, (unsigned long long)*size);
+  touch_pages(buf, *size);
   char* b = static_cast<char*>(buf);
   char* stp = b + sizeof(CheckpointHeader);
   float* tau = reinterpret_cast<float*>(stp + sizeof(IterState));
@@ -1178,6 +1179,7 @@ int aco_pool_pheromone(aco_pool_handle p, int32_t slot, float* tau) {
   if (slot < 0 || slot >= p->max_slots || !p->slots[(size_t)slot].used)
     return fail(ACO_EINVAL, "slot %d is not in use", slot);
   const PoolSlot& sl = p->slots[(size_t)slot];
+  touch_pages(tau, (size_t)sl.n * sl.n * 4);
   cudaError_t e = cudaStreamSynchronize(p->side);
   if (e == cudaSuccess)
     e = cudaMemcpy2DAsync(tau, (size_t)sl.n * 4, sl.I.tau, (size_t)sl.I.ld * 4, (size_t)sl.n * 4,
