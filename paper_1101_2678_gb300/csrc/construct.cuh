@@ -425,11 +425,12 @@ __device__ __forceinline__ void construct_ant_rule(const Instance& I, const int 
       // E's 2.5 ulp).  Only cities that pass get the logarithm and the
       // division.  Best keys below 2^-92 count as 2^-92: heavier weights than
       // 2^92 pass, whatever underflows.  (The logarithm and division for
-      // every open city took 2.58e9 warp-instructions at n = 1002, 6.29 ms.)
+      // every open city took 2.58e9 warp-instructions at n = 1002, 6.29 ms;
+      // this 2.93 ms, with the loop unrolled three or nine times 3.01 and 3.50.)
       constexpr uint32_t kInf = 0x7f800000u;
       uint32_t bkey = kInf, bj = 0xffffffffu;  // the lane's smallest key and its city
       float reach = __uint_as_float(kInf);     // best 2^32 (1 + 2^-18) over the warp
-#pragma unroll 3
+#pragma unroll 1
       for (int g = 0; g < C / 4; ++g) {
         const Philox4 x = group_draw(g);
         const uint32_t xs[4] = {x.x0, x.x1, x.x2, x.x3};
