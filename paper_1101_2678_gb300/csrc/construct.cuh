@@ -167,26 +167,30 @@ struct Seg {
 };
 
 // Cities per thread before and after the compactions of the Eq. 1 walk (see
-// construct_phased.cuh): C, then 4*ceil(C/8), 4*ceil(C/16) and 4*ceil(C/32)
-// (about C/2, C/4 and C/8 in whole 4-city groups), repeats dropped.  Adding
-// 4*ceil(3C/16), or that and 4*ceil(3C/32), measured slower at every size:
-// 0.2-2 % for one instance, 10 % for the batched step.  One warp (or
-// segment) or two warps per ant with C >= kCompactMinC compact; four warps
-// per ant never do.
-constexpr int kCompactMinC = 20;
+// construct_phased.cuh): C, then 4*ceil(C/16) and 4*ceil(C/32) (about C/4 and
+// C/8 in whole 4-city groups), repeats dropped.  A listed city costs an index
+// load and an indexed load more than a chunk's, a visited chunk city two
+// instructions, so a first compaction at C/2 loses (n = 1002 0.801 ms with
+// C/2, C/4 and C/8, 0.782 with C/4 and C/8, 0.796 with C/4 alone; n = 2392
+// 3.35, 3.24, 3.26; a step of 256 instances 14.3, 12.3, 12.4), and chunks
+// below 36 cities are not compacted at all (n = 517 0.317 ms against 0.335;
+// n = 800 0.543 against 0.552).  One warp (or segment) or two warps per ant
+// compact; four warps per ant never do.
+constexpr int kCompactMinC = 36;
 template <int C, int G>
 struct Compaction {
   static constexpr bool kOn = (G == 1 || G == 2) && C >= kCompactMinC;
+  static constexpr int kPhases = 3;
   // candidate count i: C * kSixteenths[i] / 16 rounded up to a multiple of 4
   __host__ __device__ static constexpr int raw(int i) {
-    constexpr int kSixteenths[4] = {16, 8, 4, 2};
+    constexpr int kSixteenths[kPhases] = {16, 4, 2};
     return kSixteenths[i] == 16 ? C : 4 * ((kSixteenths[i] * C + 63) / 64);
   }
   // Slot count of phase j (0 = the direct phase, C), or 0 past the last.
   __host__ __device__ static constexpr int slots(int j) {
     if (!kOn) return j == 0 ? C : 0;
     int prev = 1 << 30, k = -1;
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kPhases; ++i) {
       const int v = raw(i);
       if (v > 0 && v < prev) {
         if (++k == j) return v;

@@ -1,23 +1,21 @@
 // Tour construction by Eq. 1 (Section II; the integer roulette of reading R2),
-// for every tiling, with the unvisited cities compacted up to three times
-// along the walk where a chunk holds 20 cities or more (one or two warps, or
-// one warp segment, per ant).
+// for every tiling, with the unvisited cities compacted twice along the walk
+// where a chunk holds 36 cities or more (one or two warps, or one warp segment,
+// per ant).
 //
 // A step that handles every city of the row, visited or not, pays for the
-// visited ones too; half way through a tour that is half of the work.  The
-// walk therefore runs in up to four phases:
-//   phase 0  (at most 32*C1 unvisited cities not yet reached): lane t owns the
+// visited ones too.  The walk therefore runs in up to three phases:
+//   phase 0  (more unvisited cities than phase 1 has slots): lane t owns the
 //            contiguous chunk [tC, tC + C) of the row and skips visited cities
 //            by their tabu bits;
 //   phase 1  the unvisited cities, in ascending order, are listed in shared
-//            memory and dealt out C1 = 4*ceil(C/8) per lane (lane t takes
+//            memory and dealt out C1 = 4*ceil(C/16) per lane (lane t takes
 //            entries [t*C1, t*C1 + C1)); each step reads the entries and
 //            then their weights from the staged row through them.  A visited
 //            slot's entry is pointed at a float beside the row that stays 0,
 //            so these phases keep no tabu bits and mask nothing (entries are
 //            byte offsets for a single instance, city indices in pools);
-//   phase 2  the same with C2 = 4*ceil(C/16) per lane;
-//   phase 3  the same with C3 = 4*ceil(C/32) per lane (when smaller than C2).
+//   phase 2  the same with C2 = 4*ceil(C/32) per lane (when smaller than C1).
 // Phase p starts at the first step at which the unvisited cities fit in the
 // segment's H*Cp slots.  Every phase keeps the cities of the segment in
 // ascending order, lane after lane and slot after slot, so the first city
@@ -26,12 +24,12 @@
 // order, warp 0 first; the warps combine their totals through shared memory,
 // and the warp whose range holds the target publishes the city.  The row is
 // still staged whole (bulk copy), so the L2 bytes do not change; the
-// per-candidate work of the later steps halves, quarters and eighths.
+// per-candidate work of the last quarter and eighth of the steps shrinks.
 //
 // Construct, GB300, ms, m = n unless given: quantised 64-bit sums -> this
 // walk: n = 48 0.034 -> 0.029, n = 200 0.163 -> 0.116, n = 384 0.310 -> 0.222,
-// n = 517 0.464 -> 0.335, n = 1002 1.118 -> 0.801, n = 1500 2.13 -> 1.43,
-// n = 2392 5.05 -> 3.31, n = 4096 with m = 1024 9.02 -> 6.22.  Small instances
+// n = 517 0.464 -> 0.317, n = 1002 1.118 -> 0.782, n = 1500 2.13 -> 1.40,
+// n = 2392 5.05 -> 3.24, n = 4096 with m = 1024 9.02 -> 6.16.  Small instances
 // are bound by the step's chain (about 1500 cycles at n = 1002: the row copy
 // 500, the sums 200, the scan and the lane 280, the slot 150, the rest
 // issue), large ones also by the rows: 54.7 GB at n = 2392 take 2.7 ms at the
