@@ -15,73 +15,53 @@ namespace aco {
 // ---------------------------------------------------------------------------
 
 // Nearest-neighbour tour from city 0 (ties to the lower index), C_nn and
-// tau0 = m / C_nn.  One CTA of kNnTourThreads threads; thread t owns the
-// cities 4t + 4*kNnTourThreads*r + e (e < 4), reads them with one 16-byte
-// load per r and keeps their visited bits in a register.  Each step takes
-// the minimum of the key (d << 32 | j) (lexicographic (d, j): ties to the
-// lower index) over the unvisited cities: a warp butterfly, then the warps'
-// minima through double-buffered shared memory, one barrier per step.
-constexpr int kNnTourThreads = 256;
-constexpr int kNnTourRounds = (ACO_MAX_N + 4 * kNnTourThreads - 1) / (4 * kNnTourThreads);
-
-__global__ void __launch_bounds__(kNnTourThreads) nn_tour_kernel(Instance I) {
-  __shared__ unsigned long long wmin[2][kNnTourThreads / 32];
+// tau0 = m / C_nn.  One CTA, a chain of n steps, so a step's latency is what
+// counts: thread t of T = 256, 512 or 1024 owns the cities 4t .. 4t+3, reads
+// them with one 16-byte load and keeps their visited bits.  It keeps the first
+// of its smallest distances; the warp takes the smallest distance, then the
+// lowest index at it (two REDUX); the warps' pairs go through double-buffered
+// shared memory with one barrier, and every warp reduces them the same way.
+// aco_create_coords, GB300, ms, 64-bit keys and shuffle butterflies -> this:
+// n = 300 0.319 -> 0.254, n = 1002 0.918 -> 0.620, n = 2392 2.40 -> 1.90,
+// n = 4096 4.77 -> 3.67 (a step at n = 1002 0.45 us, its row's load most of it).
+template <int T>
+__global__ void __launch_bounds__(T) nn_tour_kernel(Instance I) {
+  constexpr int kWarps = T / 32;
+  __shared__ uint2 wmin[2][kWarps];  // (distance, index)
   const int n = I.n, ld = I.ld;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  constexpr int kWarps = kNnTourThreads / 32;
-  uint32_t visited = 0;  // bit 4r + e: city 4t + 4*kNnTourThreads*r + e
+  uint32_t open = 0;  // bit e: city 4t + e is unvisited
 #pragma unroll
-  for (int r = 0; r < kNnTourRounds; ++r)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int j = 4 * t + 4 * kNnTourThreads * r + e;
-      if (j >= n || j == 0) visited |= 1u << (4 * r + e);
-    }
+  for (int e = 0; e < 4; ++e)
+    if (4 * t + e < n && 4 * t + e != 0) open |= 1u << e;
   int cur = 0;
   long long len = 0;
   for (int s = 1; s < n; ++s) {
-    const int32_t* row = I.dist + (size_t)cur * ld;
-    int4 d4[kNnTourRounds];
+    // ld is a multiple of 4, so a 16-byte load that starts below n ends below ld
+    const int4 d4 = 4 * t < n ? *reinterpret_cast<const int4*>(I.dist + (size_t)cur * ld + 4 * t)
+                              : make_int4(0, 0, 0, 0);
+    const uint32_t dv[4] = {(uint32_t)d4.x, (uint32_t)d4.y, (uint32_t)d4.z, (uint32_t)d4.w};
+    uint32_t bd = 0xffffffffu, bj = 0xffffffffu;  // (distances are below 2^31)
 #pragma unroll
-    for (int r = 0; r < kNnTourRounds; ++r) {
-      const int j0 = 4 * t + 4 * kNnTourThreads * r;
-      // ld is a multiple of 4, so a 16-byte load that starts below n ends below ld
-      d4[r] = j0 < n ? *reinterpret_cast<const int4*>(row + j0) : make_int4(0, 0, 0, 0);
-    }
-    unsigned long long key = ~0ull;
-#pragma unroll
-    for (int r = 0; r < kNnTourRounds; ++r) {
-      const int j0 = 4 * t + 4 * kNnTourThreads * r;
-      const int dv[4] = {d4[r].x, d4[r].y, d4[r].z, d4[r].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const unsigned long long k =
-            ((unsigned long long)(uint32_t)dv[e] << 32) | (uint32_t)(j0 + e);
-        if (!((visited >> (4 * r + e)) & 1u) && k < key) key = k;
+    for (int e = 0; e < 4; ++e)
+      if (((open >> e) & 1u) && dv[e] < bd) {
+        bd = dv[e];
+        bj = (uint32_t)(4 * t + e);
       }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long other = __shfl_xor_sync(FULL, key, o);
-      key = other < key ? other : key;
-    }
-    if (lane == 0) wmin[s & 1][warp] = key;
+    uint32_t wd = __reduce_min_sync(FULL, bd);
+    uint32_t wj = __reduce_min_sync(FULL, bd == wd ? bj : 0xffffffffu);
+    if (lane == 0) wmin[s & 1][warp] = make_uint2(wd, wj);
     __syncthreads();
-    key = wmin[s & 1][0];
-#pragma unroll
-    for (int w = 1; w < kWarps; ++w) {
-      const unsigned long long other = wmin[s & 1][w];
-      key = other < key ? other : key;
-    }
-    int next = (int)(uint32_t)key;
-    if (key == ~0ull || next >= n) {  // cannot happen while a city is unvisited
+    const uint2 v = wmin[s & 1][lane % kWarps];
+    wd = __reduce_min_sync(FULL, v.x);
+    wj = __reduce_min_sync(FULL, v.x == wd ? v.y : 0xffffffffu);
+    int next = (int)wj;
+    if (wj >= (uint32_t)n) {  // cannot happen while a city is unvisited
       if (t == 0) atomicOr(&I.st->status, kStatusBadTour);
       next = 0;
     }
-    const int rel = next - 4 * t;
-    if (rel >= 0 && (rel % (4 * kNnTourThreads)) < 4)
-      visited |= 1u << (4 * (rel / (4 * kNnTourThreads)) + (rel % (4 * kNnTourThreads)));
-    len += (long long)(key >> 32);
+    if ((next >> 2) == t) open &= ~(1u << (next & 3));
+    len += (long long)wd;
     cur = next;
   }
   if (t == 0) {
@@ -483,7 +463,13 @@ static int grid_for(size_t work, int threads, int sms) {
 }
 
 cudaError_t launch_setup(const Instance& I, int sms, cudaStream_t st) {
-  nn_tour_kernel<<<1, kNnTourThreads, 0, st>>>(I);
+  static_assert(ACO_MAX_N <= 4 * 1024, "nn_tour_kernel holds four cities per thread");
+  if (I.n <= 1024)
+    nn_tour_kernel<256><<<1, 256, 0, st>>>(I);
+  else if (I.n <= 2048)
+    nn_tour_kernel<512><<<1, 512, 0, st>>>(I);
+  else
+    nn_tour_kernel<1024><<<1, 1024, 0, st>>>(I);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   init_matrices_kernel<<<grid_for((size_t)I.n * I.ld, 256, sms), 256, 0, st>>>(I);
