@@ -295,17 +295,7 @@ __device__ __forceinline__ void acs_construct_body(const Instance& I, uint32_t* 
   if (lane == 0) I.lens[k] = len;
 }
 
-// 16 bytes of a row that other warps of the CTA may be storing to: each float
-// is the value before or after the store (the caller puts the new value in).
-__device__ __forceinline__ float4 load_row4(const float* p) {
-  float4 v;
-  asm volatile("ld.relaxed.cta.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "l"(p)
-               : "memory");
-  return v;
-}
-
+// Cells that other warps of the CTA may be reading or storing to.
 __device__ __forceinline__ float load_cell(const float* p) {
   float v;
   asm volatile("ld.relaxed.cta.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
@@ -316,11 +306,17 @@ __device__ __forceinline__ void store_cell(float* p, float v) {
   asm volatile("st.relaxed.cta.global.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
 }
 
-// The same colony without lists, for n <= 128 B: each warp keeps its ant's
-// current row in registers (lane l holds cities 128 j + 4 l + e) and its tabu
-// bits in one register per eight blocks.  One colony is a chain of n lockstep
-// steps on one SM, so what counts is a step's latency:
-//  - the next row and the crossed edge's tau and eta^beta are loaded together
+// Order this thread's global stores before later bulk copies of what they wrote.
+__device__ __forceinline__ void fence_proxy_async_global() {
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+}
+
+// The same colony without lists, for n <= 128 B: each warp brings its ant's
+// current row into shared memory with one bulk copy and its registers (lane l
+// holds cities 128 j + 4 l + e), and keeps the tabu bits in one register per
+// eight blocks.  One colony is a chain of n lockstep steps on one SM, so what
+// counts is a step's latency:
+//  - the next row and the crossed edge's tau and eta^beta are fetched together
 //    as soon as the city is known, before the barriers; the few cells of the
 //    row that this step's local updates change are put in afterwards (the
 //    edges and their new choice_info are in shared memory by then);
@@ -330,14 +326,16 @@ __device__ __forceinline__ void store_cell(float* p, float v) {
 //    the target with the rounding error to spare names it (see eq1_phase in
 //    construct_phased.cuh for why that is the integer roulette's city);
 //    otherwise the step runs the integer roulette (acs_dense_choice).
-// m = 10, ms per construction, rows read again in every pass -> this kernel:
-// n = 48 0.083 -> 0.054, n = 200 0.374 -> 0.200, n = 517 1.29 -> 1.01,
-// n = 1002 3.89 -> 2.32, n = 2392 14.3 -> 11.3, n = 4096 35.8 -> 35.3.  Of a
-// step at n = 1002 (4900 cycles) about 2000 are the ten rows on their way
-// through one SM's port of the L2, 500 the crossed cell's tau and eta^beta.
+// m = 10, GB300, ms per construction, every pass over the row from L1 / rows
+// loaded by the lanes / this kernel: n = 48 0.083 / 0.054 / 0.057, n = 200
+// 0.374 / 0.200 / 0.221, n = 517 1.29 / 1.01 / 0.66, n = 1002 3.89 / 2.32 /
+// 1.42, n = 2392 14.3 / 11.3 / 5.69, n = 4096 35.8 / 35.3 / 18.1 (loads by ten
+// warps queue in the SM's load unit for 1400 cycles of a step at n = 1002); a
+// step of 256 colonies 4.59 / 2.89 / 1.82.
 template <int B>
 __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_seen,
-                                              uint32_t* s_edge, float* s_choice) {
+                                              uint32_t* s_edge, float* s_choice,
+                                              unsigned long long* s_bar, float* rows) {
   constexpr int NW = (B + 7) / 8;
   // roundings: the prefix before the lane's cities and, inside the target,
   // the whole sum (four cities, the scan, the blocks each); the lane's own
@@ -369,12 +367,17 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
     }
     if (lane == 0) seen[c >> 5] |= 1u << (c & 31);
   };
+  float* srow = rows + (size_t)k * ld;
+  const uint32_t srow_a = smem_u32(srow), bar = smem_u32(s_bar + k);
+  uint32_t parity = 0u;
+  bool waits_ok = true;
   auto load_row = [&](int c) {
-    const float* row = I.choice + (size_t)c * ld + 4 * lane;
-#pragma unroll
-    for (int j = 0; j < B; ++j)
-      v[j] = 128 * j + 4 * lane < n ? load_row4(row + 128 * j) : make_float4(0.f, 0.f, 0.f, 0.f);
+    bulk_load_if(lane == 0, srow_a, I.choice + (size_t)c * ld, (uint32_t)ld * 4u, bar);
   };
+  // cells of the row that the last step's local updates changed: the ants
+  // whose edges touch the current city, and their edges
+  unsigned touch = 0u;
+  uint32_t e = 0xffffffffu;
 
   int start = 0;
   if (active) {
@@ -382,7 +385,12 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
     __syncwarp();
     const Philox4 x0 = step_draw(I.seed, 0u, (uint32_t)k, it);
     start = (int)__umulhi(x0.x0, (uint32_t)n);
-    if (lane == 0) tour[0] = start;
+    if (lane == 0) {
+      tour[0] = start;
+      mbar_init(bar, 1);
+      fence_mbar_init();
+    }
+    __syncwarp();
     mark(start);
     load_row(start);
   }
@@ -401,6 +409,27 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
         }
         const uint32_t x1 = __shfl_sync(FULL, w1, off), x2 = __shfl_sync(FULL, w2, off);
         const bool exploit = (unsigned long long)x2 < I.acs_threshold;
+        if (!mbar_try_wait(bar, parity) && waits_ok && !mbar_wait_bounded(bar, parity)) {
+          waits_ok = false;  // stale data from here on; the status word says so
+          if (lane == 0) atomicOr(&I.st->status, kStatusTimeout);
+        }
+        parity ^= 1u;
+        if (touch) {
+          do {
+            const int i = __ffs(touch) - 1;
+            touch &= touch - 1;
+            const uint32_t ei = __shfl_sync(FULL, e, i);
+            if (lane == 0)
+              srow[(ei >> 16) == (uint32_t)cur ? ei & 0xffffu : ei >> 16] = s_choice[i];
+          } while (touch);
+          if (lane == 0) fence_proxy_async_smem();  // before the next copy into the row
+          __syncwarp();
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+          v[j] = 128 * j + 4 * lane < n
+                     ? *reinterpret_cast<const float4*>(srow + 128 * j + 4 * lane)
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
         // visited cities: below every weight, or nothing in a sum
         const float shut = exploit ? -1.0f : 0.0f;
 #pragma unroll
@@ -473,6 +502,7 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
           if (lane == 0) atomicOr(&I.st->status, kStatusBadTour);
           next = start;
         }
+        __syncwarp();  // every lane has read the row
         if (s + 1 < n) load_row(next);
         mark(next);
         if (lane == 0) tour[s] = next;
@@ -487,9 +517,9 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
     // lockstep: every ant has chosen from the same state; then the local
     // updates, once per ant that crossed the edge, stored by the first of them
     __syncthreads();
-    uint32_t e = 0xffffffffu, mine = 0u;
     if (active) {
-      mine = s_edge[k];
+      const uint32_t mine = s_edge[k];
+      e = 0xffffffffu;
       if (lane < m) e = s_edge[lane];
       const unsigned same = __ballot_sync(FULL, e == mine);
       if (lane == 0) {
@@ -502,34 +532,14 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
           store_cell(I.tau + hi * ld + lo, t);
           store_cell(I.choice + lo * ld + hi, ch);
           store_cell(I.choice + hi * ld + lo, ch);
+          fence_proxy_async_global();
         }
       }
+      // (the ant's own edge leads to a visited city)
+      touch = __ballot_sync(FULL, lane < m && e != mine &&
+                                      ((e >> 16) == (uint32_t)next || (e & 0xffffu) == (uint32_t)next));
     }
     __syncthreads();
-    if (active) {
-      // cells of the new row that this step changed (the ant's own edge leads
-      // to a visited city)
-      const uint32_t lo = e >> 16, hi = e & 0xffffu;
-      unsigned touch = __ballot_sync(FULL, lane < m && e != mine &&
-                                               (lo == (uint32_t)next || hi == (uint32_t)next));
-      while (touch) {
-        const int i = __ffs(touch) - 1;
-        touch &= touch - 1;
-        const uint32_t ei = __shfl_sync(FULL, e, i);
-        const int c = (int)((ei >> 16) == (uint32_t)next ? ei & 0xffffu : ei >> 16);
-        const float ch = s_choice[i];
-        if (lane == ((c >> 2) & 31)) {
-#pragma unroll
-          for (int j = 0; j < B; ++j)
-            if (j == (c >> 7)) {
-              if ((c & 3) == 0) v[j].x = ch;
-              if ((c & 3) == 1) v[j].y = ch;
-              if ((c & 3) == 2) v[j].z = ch;
-              if ((c & 3) == 3) v[j].w = ch;
-            }
-        }
-      }
-    }
     cur = next;
   }
   if (!active) return;
@@ -549,19 +559,24 @@ constexpr int kAcsRowThreads = B <= 4 ? 1024 : (B <= 8 ? 512 : 320);
 
 template <int B>
 __global__ void __launch_bounds__(kAcsRowThreads<B>, 1) acs_rows_kernel(Instance I) {
-  extern __shared__ uint32_t acs_seen[];
+  extern __shared__ __align__(16) float acs_rows[];  // a row per ant, then the tabu bitmaps
   __shared__ uint32_t s_edge[32];
   __shared__ float s_choice[32];
-  acs_rows_body<B>(I, acs_seen, s_edge, s_choice);
+  __shared__ unsigned long long s_bar[32];
+  acs_rows_body<B>(I, reinterpret_cast<uint32_t*>(acs_rows + (size_t)I.m * I.ld), s_edge, s_choice,
+                   s_bar, acs_rows);
 }
 
 template <int B>
 __global__ void __launch_bounds__(kAcsRowThreads<B>, 1)
     acs_rows_slots_kernel(const Instance* __restrict__ insts, const int* __restrict__ slots) {
-  extern __shared__ uint32_t acs_seen[];
+  extern __shared__ __align__(16) float acs_rows[];  // a row per ant, then the tabu bitmaps
   __shared__ uint32_t s_edge[32];
   __shared__ float s_choice[32];
-  acs_rows_body<B>(insts[slots[blockIdx.x]], acs_seen, s_edge, s_choice);
+  __shared__ unsigned long long s_bar[32];
+  const Instance& I = insts[slots[blockIdx.x]];
+  acs_rows_body<B>(I, reinterpret_cast<uint32_t*>(acs_rows + (size_t)I.m * I.ld), s_edge, s_choice,
+                   s_bar, acs_rows);
 }
 
 template <bool kNN>
@@ -639,17 +654,44 @@ cudaError_t launch_acs_init(const Instance& I, int sms, cudaStream_t st) {
 // than 10), and the row is read again in every pass instead.
 using AcsBlocks = ChunkList<1, 2, 4, 6, 8, 12, 16, 20, 24, 32>;
 
+// Shared memory of a colony of up to m ants and n cities.
+static size_t acs_rows_bytes(int n, int m) {
+  return (size_t)m * (((size_t)n + 3) / 4 * 4 * sizeof(float) +
+                      ((size_t)n + 31) / 32 * sizeof(uint32_t));
+}
+
+constexpr size_t kAcsRowsMost = 224 * 1024;
+
+template <int B, bool kSlots>
+static bool acs_rows_ready() {
+  static std::atomic<unsigned long long> done{0};
+  return once_per_device(done, [] {
+           if constexpr (kSlots)
+             return cudaFuncSetAttribute(acs_rows_slots_kernel<B>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kAcsRowsMost);
+           else
+             return cudaFuncSetAttribute(acs_rows_kernel<B>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kAcsRowsMost);
+         }) == cudaSuccess;
+}
+
 template <int... Bs>
-static bool launch_acs_rows(ChunkList<Bs...>, const Instance& I, size_t smem, cudaStream_t st) {
-  return ((I.n <= 128 * Bs && 32 * I.m <= kAcsRowThreads<Bs> &&
+static bool launch_acs_rows(ChunkList<Bs...>, const Instance& I, cudaStream_t st) {
+  const size_t smem = acs_rows_bytes(I.n, I.m);
+  return smem <= kAcsRowsMost &&
+         ((I.n <= 128 * Bs && 32 * I.m <= kAcsRowThreads<Bs> && acs_rows_ready<Bs, false>() &&
            (acs_rows_kernel<Bs><<<1, 32 * I.m, smem, st>>>(I), true)) ||
           ...);
 }
 
 template <int... Bs>
 static bool launch_acs_rows_slots(ChunkList<Bs...>, const Instance* insts, const int* slots,
-                                  int count, int max_m, int max_n, size_t smem, cudaStream_t st) {
-  return ((max_n <= 128 * Bs && 32 * max_m <= kAcsRowThreads<Bs> &&
+                                  int count, int max_m, int max_n, cudaStream_t st) {
+  const size_t smem = acs_rows_bytes(max_n, max_m);
+  return smem <= kAcsRowsMost &&
+         ((max_n <= 128 * Bs && 32 * max_m <= kAcsRowThreads<Bs> && acs_rows_ready<Bs, true>() &&
            (acs_rows_slots_kernel<Bs><<<count, 32 * max_m, smem, st>>>(insts, slots), true)) ||
           ...);
 }
@@ -659,7 +701,7 @@ cudaError_t launch_acs_construct(const Instance& I, cudaStream_t st) {
   const size_t smem = (size_t)I.m * ((I.n + 31) / 32) * sizeof(uint32_t);
   if (I.nn > 0)
     acs_construct_kernel<true><<<1, 32 * I.m, smem, st>>>(I);
-  else if (!launch_acs_rows(AcsBlocks{}, I, smem, st))
+  else if (!launch_acs_rows(AcsBlocks{}, I, st))
     acs_construct_kernel<false><<<1, 32 * I.m, smem, st>>>(I);
   return cudaGetLastError();
 }
@@ -676,7 +718,7 @@ cudaError_t launch_acs_construct_slots(const Instance* insts, const int* slots, 
   const size_t smem = (size_t)max_m * ((max_n + 31) / 32) * sizeof(uint32_t);
   if (lists)
     acs_construct_slots_kernel<true><<<count, 32 * max_m, smem, st>>>(insts, slots);
-  else if (!launch_acs_rows_slots(AcsBlocks{}, insts, slots, count, max_m, max_n, smem, st))
+  else if (!launch_acs_rows_slots(AcsBlocks{}, insts, slots, count, max_m, max_n, st))
     acs_construct_slots_kernel<false><<<count, 32 * max_m, smem, st>>>(insts, slots);
   return cudaGetLastError();
 }
