@@ -472,15 +472,15 @@ def run_ours(args, w, rank, world, local):
         return
     peaks, peak_kind = measured_peaks()
     if args.variant == "acs":
-        kernel = "acs_construct_kernel"
+        kernel = "acs_rows_kernel"
     elif args.nn:
         kernel = "construct_nn_kernel"
-    elif args.selection == "eq1" and tiling[0] == 1 and n > 12 * tiling[2]:
-        # one warp or segment per ant with at least 20 cities per lane: the
-        # walk with compaction
-        kernel = "construct_phased_kernel"
+    elif args.selection != "eq1":
+        kernel = "construct_rule_kernel"
+    elif n <= 240 and not (args.lanes_per_ant or args.warps_per_ant or args.ants_per_cta):
+        kernel = "construct_small_kernel"  # the whole matrix in shared memory
     else:
-        kernel = "construct_kernel"
+        kernel = "construct_phased_kernel"
     l2 = measure_l2_read_gbs()
     roof = construct_roofline(n, m, con_ms, l2, peaks, peak_kind, kernel=kernel, nn=args.nn)
     if not (args.nn or args.selection != "eq1" or args.lanes_per_ant or args.warps_per_ant

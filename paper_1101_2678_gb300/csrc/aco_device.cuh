@@ -185,11 +185,6 @@ __device__ __forceinline__ int exponent_of_bits(uint32_t b) {
 // 2^e as a float, for -126 <= e <= 127.
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
-// 2^e as a double, for -1022 <= e <= 1023.
-__device__ __forceinline__ double pow2d(int e) {
-  return __longlong_as_double((long long)(e + 1023) << 52);
-}
-
 // floor(d * 2^shift) for a float d >= 0 by its significand (the FP64 units are
 // few: a conversion there costs as much as a warp's whole integer shift).
 __device__ __forceinline__ unsigned long long fixed_of(float d, int shift) {

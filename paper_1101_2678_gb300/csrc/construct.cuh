@@ -203,7 +203,9 @@ struct Compaction {
 
 // Shared memory of one ant group: the staged row (H*G*C floats, 16-byte
 // aligned), its mbarrier, and (when the walk compacts) the list of unvisited
-// cities, up to H * 4*ceil(C/8) 16-bit entries.
+// cities, up to H*G * 4*ceil(C/16) 16-bit entries.  (Rows of ld floats would
+// leave room for more ants, but a group stride known only at run time made the
+// compacting walk 10-30 % slower: n = 2392 3.34 -> 4.31 ms.)
 template <int C, int G, int H>
 struct StageLayout {
   static constexpr int kRowFloats = H * G * C;
@@ -569,10 +571,10 @@ __global__ void __launch_bounds__(256) construct_rule_kernel(Instance I) {
 // (or two warps) per ant.  Its phases are inlined into one body; without a
 // ceiling the register allocator hoists the row's loads.  The ceilings were
 // chosen by measurement on the GB300: 64 up to C = 36, where the shared
-// memory of a row leaves room for 32 ants an SM (n = 1002, m = 4864: 1.58 ms
-// against 1.98 at 72; a step of 256 instances 14.3 ms against 14.5; 48 and 56
-// are 1-2 % slower everywhere); above, the rows limit the ants and 128 costs
-// nothing (n = 2392 3.30 ms; 96: 3.32, 72: 3.34).
+// memory of a row leaves room for 32 ants an SM (with lists at C/2 still: n =
+// 1002, m = 4864 1.58 ms against 1.98 at 72, a step of 256 instances 14.3 ms
+// against 14.5; 48 and 56 are 1-2 % slower everywhere); above, the rows limit
+// the ants and 128 costs nothing (n = 2392 3.30 ms; 96: 3.32, 72: 3.34).
 // Two warps per ant (n > 2432) would hold 2 x 13 warps at C = 52 and 2 x 11 at
 // C = 60 by their rows: ceilings that let them all reside (n = 3100 11.6 ms at
 // 128, 9.73 at 72).
