@@ -470,10 +470,12 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
         for (int wd = 0; wd < NW; ++wd)
           if (wd == (li >> 5)) vis[wd] |= 1u << (li & 31);
       }
-    } else if (tg == got.chosen) {
-      // every read of this entry in this step came before the shuffle (or
-      // barrier) that decided it
-      ulist[tg * CP + got.slot] = (uint16_t)kZeroEntry;
+    } else {
+      // Every lane of the chosen thread's warp (or segment) read this entry to
+      // decide: they all have to be past those reads before it changes.  (With
+      // several warps per ant the barrier that published the city says so.)
+      if constexpr (G == 1) seg.sync();
+      if (tg == got.chosen) ulist[tg * CP + got.slot] = (uint16_t)kZeroEntry;
     }
     if (tg == 0) tour[s] = next;
     w.cur = next;
