@@ -591,6 +591,10 @@ __device__ __forceinline__ void construct_ant_phased(const Instance& I, const in
     srow[StageLayout<C, G, H>::kZeroSlot] = 0.0f;  // the weight of a visited list slot
     if (G > 1) gs->fnext[0] = gs->fnext[1] = -1;
   }
+  // In a persistent launch the ant before may have staged its rows by lane
+  // copies (generic proxy) in these bytes: each lane orders its own before the
+  // bulk copies that follow the group's wait.
+  fence_proxy_async_smem();
   group_wait();
 
   WalkState w{start, 1, 0, 0.0f, 0u, true};

@@ -79,3 +79,17 @@ def test_walk_in_any_order(orc, emulate, c, g, h, n, beta, lane_copy):
     rc, tours, lens, _ = emulate(c, g, h, choice, dist, ants, [lane_copy] * 2, 5, n)
     assert rc == 0
     assert np.array_equal(tours, want[0]) and np.array_equal(lens, want[1])
+
+
+# A persistent launch builds one ant after another in the same shared memory, and classes may
+# differ in their row staging: every thread that copied rows itself has to fence its writes before
+# the copy engine writes there.
+@pytest.mark.parametrize("c,g,h,n", [(36, 1, 32, 120), (12, 1, 32, 100), (36, 1, 8, 90),
+                                     (36, 2, 32, 200)])
+def test_bulk_copy_after_lane_copies_is_fenced(orc, emulate, c, g, h, n):
+    dist, choice = _instance(orc, n)
+    ants = 2 * (32 // h)
+    want = orc.construct(choice, dist, ants, seed=9, iteration=0)
+    rc, tours, lens, unfenced = emulate(c, g, h, choice, dist, ants, [1, 0], 9, n)
+    assert rc == 0 and np.array_equal(tours, want[0]) and np.array_equal(lens, want[1])
+    assert unfenced == 0
