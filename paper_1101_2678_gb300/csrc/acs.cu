@@ -370,9 +370,9 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
   float* srow = rows + (size_t)k * ld;
   const uint32_t srow_a = smem_u32(srow), bar = smem_u32(s_bar + k);
   uint32_t parity = 0u;
-  bool waits_ok = true;
+  int role = lane;  // 0 issues the copies; -2 minus the parity of a wait that gave up
   auto load_row = [&](int c) {
-    bulk_load_if(lane == 0, srow_a, I.choice + (size_t)c * ld, (uint32_t)ld * 4u, bar);
+    bulk_load_if(role == 0, srow_a, I.choice + (size_t)c * ld, (uint32_t)ld * 4u, bar);
   };
   // cells of the row that the last step's local updates changed: the ants
   // whose edges touch the current city, and their edges
@@ -409,9 +409,10 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
         }
         const uint32_t x1 = __shfl_sync(FULL, w1, off), x2 = __shfl_sync(FULL, w2, off);
         const bool exploit = (unsigned long long)x2 < I.acs_threshold;
-        if (!mbar_try_wait(bar, parity) && waits_ok && !mbar_wait_bounded(bar, parity)) {
-          waits_ok = false;  // stale data from here on; the status word says so
-          if (lane == 0) atomicOr(&I.st->status, kStatusTimeout);
+        if (!mbar_try_wait(bar, parity) && role >= 0 && !mbar_wait_bounded(bar, parity)) {
+          // stale data and no further copies from here on; the status word says so
+          role = -2 - (int)parity;
+          atomicOr(&I.st->status, kStatusTimeout);
         }
         parity ^= 1u;
         if (touch) {
@@ -543,6 +544,8 @@ __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_s
     cur = next;
   }
   if (!active) return;
+  // the copy in flight, again with a limit
+  if (role < 0) mbar_wait_bounded(bar, (uint32_t)role & 1u);
   if (lane == 0) tour[n] = start;
   __syncwarp();
   long long len = 0;

@@ -314,7 +314,7 @@ __device__ __forceinline__ void construct_ant_rule(const Instance& I, const int 
   const uint32_t bar = srow_a + (uint32_t)StageLayout<C, G, H>::kRowFloats * 4u;
   const uint32_t row_bytes = (uint32_t)ld * 4u;
   uint32_t phase = 0;
-  bool waits_ok = true;
+  int role = tg;  // 0 issues the copies; -2 minus the parity of a wait that gave up
   if (tg == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
@@ -331,10 +331,11 @@ __device__ __forceinline__ void construct_ant_rule(const Instance& I, const int 
       for (int i = tg; i < (ld >> 2); i += NT) dst[i] = src[i];
       group_wait();
     } else {
-      bulk_load_if(tg == 0, srow_a, choice + (size_t)cur * ld, row_bytes, bar);
-      if (!mbar_try_wait(bar, phase) && waits_ok && !mbar_wait_bounded(bar, phase)) {
-        waits_ok = false;  // stale data from here on; the status word says so
-        if (tg == 0) atomicOr(&I.st->status, kStatusTimeout);
+      bulk_load_if(role == 0, srow_a, choice + (size_t)cur * ld, row_bytes, bar);
+      if (!mbar_try_wait(bar, phase) && role >= 0 && !mbar_wait_bounded(bar, phase)) {
+        // stale data and no further copies from here on; the status word says so
+        role = -2 - (int)phase;
+        atomicOr(&I.st->status, kStatusTimeout);
       }
       phase ^= 1u;
     }
@@ -509,6 +510,8 @@ __device__ __forceinline__ void construct_ant_rule(const Instance& I, const int 
     cur = next;
     group_wait();
   }
+  // the copy in flight, again with a limit
+  if (role < 0) mbar_wait_bounded(bar, (uint32_t)role & 1u);
   if (tg == 0) tour[n] = start;
   group_wait();
 

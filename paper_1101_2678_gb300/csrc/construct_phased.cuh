@@ -54,7 +54,10 @@ struct WalkState {
   int live;      // unvisited cities listed for the current phase (gather phases)
   float u;       // this lane's uniform r / 2^64 for its step of the window
   uint32_t parity;          // mbarrier phase of the row copy
-  bool waits_ok;
+  // The thread's index in the group (0 issues the copies), or, after a wait that
+  // gave up, -2 minus the parity it waited for.  (One value for both: a flag of
+  // its own in the issue condition cost the walk 1 %.)
+  int role;
 };
 
 // The city of one step: `next`, and in gather phases the thread and slot that
@@ -291,7 +294,7 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
                       src + 4 * i * NT);
       cp_async_wait_all();
     } else {
-      bulk_load_if(tg == 0, srow_a, choice + (size_t)cur * ld, row_bytes, bar);
+      bulk_load_if(w.role == 0, srow_a, choice + (size_t)cur * ld, row_bytes, bar);
     }
     const int off = (s - 1) % H;
     if (off == 0) {
@@ -302,9 +305,10 @@ __device__ __forceinline__ void eq1_phase(const Instance& I, const int ant, cons
     if constexpr (kLane) {
       group_wait();
     } else {
-      if (!mbar_try_wait(bar, w.parity) && w.waits_ok && !mbar_wait_bounded(bar, w.parity)) {
-        w.waits_ok = false;  // stale data from here on; the status word says so
-        if (tg == 0) atomicOr(&I.st->status, kStatusTimeout);
+      if (!mbar_try_wait(bar, w.parity) && w.role >= 0 && !mbar_wait_bounded(bar, w.parity)) {
+        // stale data and no further copies from here on; the status word says so
+        w.role = -2 - (int)w.parity;
+        atomicOr(&I.st->status, kStatusTimeout);
       }
       w.parity ^= 1u;
     }
@@ -561,9 +565,11 @@ __device__ __forceinline__ void eq1_phases(const Instance& I, const int ant, con
 }
 
 // The whole walk of one ant (G warps or one H-lane segment) and its length
-// and neighbour buckets.
+// and neighbour buckets.  False where this thread's wait for a row gave up: the
+// staging memory may still have a copy in flight, and no further bulk copy may
+// use it.
 template <int C, int G, int H, bool kPool>
-__device__ __forceinline__ void construct_ant_phased(const Instance& I, const int ant,
+__device__ __forceinline__ bool construct_ant_phased(const Instance& I, const int ant,
                                                      const int tg, const Seg<H> seg,
                                                      GroupSmem* gs, const int bar_id, float* srow,
                                                      const bool lane_copy) {
@@ -586,8 +592,10 @@ __device__ __forceinline__ void construct_ant_phased(const Instance& I, const in
   if (tg == 0) tour[0] = start;
   const uint32_t bar = smem_u32(srow) + (uint32_t)StageLayout<C, G, H>::kRowFloats * 4u;
   if (tg == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
+    if (!lane_copy) {
+      mbar_init(bar, 1);
+      fence_mbar_init();
+    }
     srow[StageLayout<C, G, H>::kZeroSlot] = 0.0f;  // the weight of a visited list slot
     if (G > 1) gs->fnext[0] = gs->fnext[1] = -1;
   }
@@ -597,11 +605,13 @@ __device__ __forceinline__ void construct_ant_phased(const Instance& I, const in
   fence_proxy_async_smem();
   group_wait();
 
-  WalkState w{start, 1, 0, 0.0f, 0u, true};
+  WalkState w{start, 1, 0, 0.0f, 0u, tg};
   if (lane_copy)
     eq1_phases<C, G, H, kPool, true, 0>(I, ant, tg, seg, gs, bar_id, srow, ulist, start, w);
   else
     eq1_phases<C, G, H, kPool, false, 0>(I, ant, tg, seg, gs, bar_id, srow, ulist, start, w);
+  // the copy in flight, again with a limit
+  if (w.role < 0) mbar_wait_bounded(bar, (uint32_t)w.role & 1u);
   if (tg == 0) tour[n] = start;
   group_wait();
 
@@ -623,6 +633,7 @@ __device__ __forceinline__ void construct_ant_phased(const Instance& I, const in
     for (int k = 0; k < G; ++k) len += gs->wlen[k];
   }
   if (tg == 0) I.lens[ant] = len;
+  return w.role >= 0;
 }
 
 }  // namespace aco

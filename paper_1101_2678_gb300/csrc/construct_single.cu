@@ -19,6 +19,11 @@ namespace {
 constexpr int kSingleWarps = 4;
 constexpr int kSingleBytes = StageLayout<36, 1, 32>::kBytes;  // the widest chunk handled
 
+template <int C>
+struct Width {
+  static constexpr int value = C;
+};
+
 __global__ void __maxnreg__(64)
     construct_single_kernel(const Instance* __restrict__ insts, const int2* __restrict__ items,
                             SingleClasses cls, int total, int* ticket) {
@@ -27,6 +32,7 @@ __global__ void __maxnreg__(64)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* srow = reinterpret_cast<float*>(stage + warp * kSingleBytes);
   const Seg<32> seg(lane);
+  bool ok = true;
   for (;;) {
     int t = 0;
     if (lane == 0) t = atomicAdd(ticket, 1);
@@ -39,27 +45,24 @@ __global__ void __maxnreg__(64)
     }
     const int2 it = items[cls.begin[k] + idx];
     const Instance& I = insts[it.x];
-    const bool lc = cls.lane_copy[k] != 0;
+    // after a wait of this warp gave up: no more bulk copies, and every result
+    // from its staging memory is marked
+    const bool lc = cls.lane_copy[k] != 0 || !ok;
+    if (!ok && lane == 0) atomicOr(&I.st->status, kStatusTimeout);
+    bool waited = true;
+    auto build = [&](auto width) {
+      waited = construct_ant_phased<decltype(width)::value, 1, 32, true>(
+          I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
+    };
     switch (cls.C[k]) {
-      case 4:
-        construct_ant_phased<4, 1, 32, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
-        break;
-      case 12:
-        construct_ant_phased<12, 1, 32, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
-        break;
-      case 20:
-        construct_ant_phased<20, 1, 32, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
-        break;
-      case 28:
-        construct_ant_phased<28, 1, 32, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
-        break;
-      case 36:
-        construct_ant_phased<36, 1, 32, true>(I, it.y, lane, seg, &gs[warp], 1 + warp, srow, lc);
-        break;
-      default:
-        break;
+      case 4: build(Width<4>{}); break;
+      case 12: build(Width<12>{}); break;
+      case 20: build(Width<20>{}); break;
+      case 28: build(Width<28>{}); break;
+      case 36: build(Width<36>{}); break;
+      default: break;
     }
-    __syncwarp();
+    ok = __all_sync(FULL, waited) && ok;
   }
 }
 

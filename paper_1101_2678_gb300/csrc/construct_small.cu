@@ -65,7 +65,10 @@ __global__ void __launch_bounds__(1024) construct_small_kernel(Instance I) {
     const Philox4 x0 = step_draw(seed, 0u, (uint32_t)ant, iter);
     start = (int)__umulhi(x0.x0, (uint32_t)n);
   }
-  if (!mbar_wait_bounded(bar, 0u) && lane == 0) atomicOr(&I.st->status, kStatusTimeout);
+  // (twice the limit: the CTA goes on to its end with the copy in flight if it
+  // still has not come)
+  if (!mbar_wait_bounded(bar, 0u, 2 * kWaitPolls) && lane == 0)
+    atomicOr(&I.st->status, kStatusTimeout);
   if (ant >= I.m) return;
 
   const Seg<32> seg(lane);

@@ -4,7 +4,7 @@
 // synchronisations, so a result that needs the lanes of a warp to keep in step comes out wrong here.
 //
 // Also recorded: bulk copies (async proxy) into bytes that a thread wrote through the generic
-// proxy without a proxy fence since (cp.async rows).
+// proxy without a proxy fence since (cp.async rows), and copies that follow one that never came.
 #include <ucontext.h>
 
 #include <bit>
@@ -38,6 +38,7 @@ struct Fibre {
 };
 struct Mbar {
   unsigned phase = 0;
+  bool stuck = false;
 };
 
 static std::vector<Fibre> fibres;
@@ -45,7 +46,7 @@ static ucontext_t home;
 static int self;
 static uint3 tid;
 static bool broken;  // lanes of one group met at different collectives, or none can go on
-static int unfenced;
+static int unfenced, late, copies, stall;
 static std::map<std::pair<int, unsigned>, Group> groups;
 static std::map<uint32_t, Mbar> mbars;
 alignas(16) static unsigned char smem[1 << 18];
@@ -208,9 +209,9 @@ inline bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return false;
 }
 inline bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < 100000; ++i)
+  for (int i = 0; i < (emu::mbars[bar].stuck ? 50 : 100000); ++i)
     if (mbar_try_wait(bar, parity)) return true;
-  emu::broken = true;
+  if (!emu::mbars[bar].stuck) emu::broken = true;
   return false;
 }
 inline void fence_mbar_init() {}
@@ -226,6 +227,9 @@ inline bool in_source(const void* src, uint32_t bytes) {
 }
 inline void bulk_load_if(bool go, uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   if (!go) return;
+  if (emu::mbars[bar].stuck) ++emu::late;
+  if (emu::copies++ == emu::stall) emu::mbars[bar].stuck = true;
+  if (emu::mbars[bar].stuck) return;
   for (uint32_t b = dst; b < dst + bytes; ++b)
     if (emu::writer[b]) {
       ++emu::unfenced;
@@ -273,11 +277,12 @@ void (*entry)();
 }  // namespace
 
 // Tours and lengths of `ants` ants; lane_copy[r]: row staging of the ants of round r, which share
-// shared memory with the round before.  Returns 0, or 1 where threads parted for good; *unfenced
-// counts bulk copies over generic-proxy writes without a fence.
+// shared memory with the round before; stall: the bulk copy of that number never arrives (-1: all
+// do).  Returns 0, or 1 where threads parted for good.  counts: bulk copies over generic-proxy
+// writes without a fence; copies issued on a barrier after one that never came; status bits.
 extern "C" int emulate_walk(int C, int G, int H, int n, int ants, const int* lane_copy,
                             const float* choice, const int* dist, unsigned long long seed,
-                            unsigned schedule, int* tours, long long* lens, int* unfenced) {
+                            unsigned schedule, int stall, int* tours, long long* lens, int* counts) {
   using namespace emu;
   entry = C == 36 && G == 1 && H == 32   ? thread_main<36, 1, 32>
           : C == 36 && G == 1 && H == 16 ? thread_main<36, 1, 16>
@@ -318,7 +323,8 @@ extern "C" int emulate_walk(int C, int G, int H, int n, int ants, const int* lan
   groups.clear();
   mbars.clear();
   broken = false;
-  emu::unfenced = 0;
+  unfenced = late = copies = 0;
+  emu::stall = stall;
   const int threads = G * 32;
   fibres = std::vector<Fibre>(threads);
   for (auto& f : fibres) {
@@ -350,6 +356,8 @@ extern "C" int emulate_walk(int C, int G, int H, int n, int ants, const int* lan
     tid = uint3{(unsigned)self, 0u, 0u};
     swapcontext(&home, &fibres[self].ctx);
   }
-  *unfenced = emu::unfenced;
-  return broken || st.status ? 1 : 0;
+  counts[0] = unfenced;
+  counts[1] = late;
+  counts[2] = st.status;
+  return broken ? 1 : 0;
 }

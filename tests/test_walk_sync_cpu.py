@@ -45,15 +45,15 @@ def emulate(tmp_path_factory):
                     os.path.join(HERE, "host_warp", "walk_emulator.cpp"), "-o", str(so)], check=True)
     lib = C.CDLL(str(so))
 
-    def run(c, g, h, choice, dist, ants, lane_copy, seed, schedule):
+    def run(c, g, h, choice, dist, ants, lane_copy, seed, schedule, stall=-1):
         n = dist.shape[0]
         tours, lens = np.zeros((ants, n + 1), np.int32), np.zeros(ants, np.int64)
         lane_copy = np.asarray(lane_copy, np.int32)
-        unfenced = C.c_int(0)
+        counts = np.zeros(3, np.int32)
         p = lambda x: x.ctypes.data_as(C.c_void_p)  # noqa: E731
         rc = lib.emulate_walk(c, g, h, n, ants, p(lane_copy), p(choice), p(dist),
-                              C.c_ulonglong(seed), schedule, p(tours), p(lens), C.byref(unfenced))
-        return rc, tours, lens, unfenced.value
+                              C.c_ulonglong(seed), schedule, stall, p(tours), p(lens), p(counts))
+        return rc, tours, lens, counts
     return run
 
 
@@ -76,8 +76,8 @@ def test_walk_in_any_order(orc, emulate, c, g, h, n, beta, lane_copy):
     dist, choice = _instance(orc, n, beta)
     ants = 32 // h + 1
     want = orc.construct(choice, dist, ants, seed=5, iteration=0)
-    rc, tours, lens, _ = emulate(c, g, h, choice, dist, ants, [lane_copy] * 2, 5, n)
-    assert rc == 0
+    rc, tours, lens, counts = emulate(c, g, h, choice, dist, ants, [lane_copy] * 2, 5, n)
+    assert rc == 0 and counts[2] == 0
     assert np.array_equal(tours, want[0]) and np.array_equal(lens, want[1])
 
 
@@ -90,6 +90,19 @@ def test_bulk_copy_after_lane_copies_is_fenced(orc, emulate, c, g, h, n):
     dist, choice = _instance(orc, n)
     ants = 2 * (32 // h)
     want = orc.construct(choice, dist, ants, seed=9, iteration=0)
-    rc, tours, lens, unfenced = emulate(c, g, h, choice, dist, ants, [1, 0], 9, n)
+    rc, tours, lens, counts = emulate(c, g, h, choice, dist, ants, [1, 0], 9, n)
     assert rc == 0 and np.array_equal(tours, want[0]) and np.array_equal(lens, want[1])
-    assert unfenced == 0
+    assert counts[0] == 0 and counts[2] == 0
+
+
+# A copy that never arrives: the wait gives up and the status says so; no copy is issued after it
+# (the shared memory goes away at the CTA's end), and the tour is still one.
+@pytest.mark.parametrize("c,g,h,n", [(36, 1, 32, 450), (36, 1, 8, 90), (36, 2, 32, 200),
+                                     (12, 1, 32, 100)])
+def test_no_copies_after_a_wait_gave_up(orc, emulate, c, g, h, n):
+    dist, choice = _instance(orc, n)
+    ants = 32 // h
+    rc, tours, _, counts = emulate(c, g, h, choice, dist, ants, [0], 7, n, stall=n // 2)
+    assert rc == 0 and counts[2] == 1
+    assert counts[1] == 0
+    assert all(sorted(t[:-1]) == list(range(n)) and t[-1] == t[0] for t in tours)
