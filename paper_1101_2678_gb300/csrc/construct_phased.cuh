@@ -633,6 +633,10 @@ __device__ __forceinline__ bool construct_ant_phased(const Instance& I, const in
     for (int k = 0; k < G; ++k) len += gs->wlen[k];
   }
   if (tg == 0) I.lens[ant] = len;
+  // In a persistent launch the warp's next ant, of this class or another, uses
+  // these bytes for its row or its own barrier.  (Initialised again while alive,
+  // the barrier's first wait timed out there, beside classes with lane copies.)
+  if (tg == 0 && !lane_copy && w.role >= 0) mbar_inval(bar);
   return w.role >= 0;
 }
 

@@ -46,7 +46,7 @@ static ucontext_t home;
 static int self;
 static uint3 tid;
 static bool broken;  // lanes of one group met at different collectives, or none can go on
-static int unfenced, late, copies, stall;
+static int unfenced, late, reused, copies, stall;
 static std::map<std::pair<int, unsigned>, Group> groups;
 static std::map<uint32_t, Mbar> mbars;
 alignas(16) static unsigned char smem[1 << 18];
@@ -184,6 +184,7 @@ inline int atomicOr(int* p, int v) {
 
 // The PTX helpers: their names are taken from the header, and the host's stand in for them.
 #define mbar_init ptx_mbar_init
+#define mbar_inval ptx_mbar_inval
 #define mbar_try_wait ptx_mbar_try_wait
 #define mbar_wait_bounded ptx_mbar_wait_bounded
 #define fence_mbar_init ptx_fence_mbar_init
@@ -193,6 +194,7 @@ inline int atomicOr(int* p, int v) {
 #define cp_async_wait_all ptx_cp_async_wait_all
 #include "aco_device.cuh"
 #undef mbar_init
+#undef mbar_inval
 #undef mbar_try_wait
 #undef mbar_wait_bounded
 #undef fence_mbar_init
@@ -202,7 +204,11 @@ inline int atomicOr(int* p, int v) {
 #undef cp_async_wait_all
 
 namespace aco {
-inline void mbar_init(uint32_t bar, uint32_t) { emu::mbars[bar] = emu::Mbar{}; }
+inline void mbar_init(uint32_t bar, uint32_t) {
+  if (emu::mbars.count(bar)) ++emu::reused;
+  emu::mbars[bar] = emu::Mbar{};
+}
+inline void mbar_inval(uint32_t bar) { emu::mbars.erase(bar); }
 inline bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   if ((emu::mbars[bar].phase & 1u) != parity) return true;
   emu::yield();
@@ -279,7 +285,8 @@ void (*entry)();
 // Tours and lengths of `ants` ants; lane_copy[r]: row staging of the ants of round r, which share
 // shared memory with the round before; stall: the bulk copy of that number never arrives (-1: all
 // do).  Returns 0, or 1 where threads parted for good.  counts: bulk copies over generic-proxy
-// writes without a fence; copies issued on a barrier after one that never came; status bits.
+// writes without a fence; copies issued on a barrier after one that never came; status bits;
+// barriers initialised again without having been invalidated.
 extern "C" int emulate_walk(int C, int G, int H, int n, int ants, const int* lane_copy,
                             const float* choice, const int* dist, unsigned long long seed,
                             unsigned schedule, int stall, int* tours, long long* lens, int* counts) {
@@ -323,7 +330,7 @@ extern "C" int emulate_walk(int C, int G, int H, int n, int ants, const int* lan
   groups.clear();
   mbars.clear();
   broken = false;
-  unfenced = late = copies = 0;
+  unfenced = late = reused = copies = 0;
   emu::stall = stall;
   const int threads = G * 32;
   fibres = std::vector<Fibre>(threads);
@@ -359,5 +366,6 @@ extern "C" int emulate_walk(int C, int G, int H, int n, int ants, const int* lan
   counts[0] = unfenced;
   counts[1] = late;
   counts[2] = st.status;
+  counts[3] = reused;
   return broken ? 1 : 0;
 }

@@ -49,7 +49,7 @@ def emulate(tmp_path_factory):
         n = dist.shape[0]
         tours, lens = np.zeros((ants, n + 1), np.int32), np.zeros(ants, np.int64)
         lane_copy = np.asarray(lane_copy, np.int32)
-        counts = np.zeros(3, np.int32)
+        counts = np.zeros(4, np.int32)
         p = lambda x: x.ctypes.data_as(C.c_void_p)  # noqa: E731
         rc = lib.emulate_walk(c, g, h, n, ants, p(lane_copy), p(choice), p(dist),
                               C.c_ulonglong(seed), schedule, stall, p(tours), p(lens), p(counts))
@@ -106,3 +106,16 @@ def test_no_copies_after_a_wait_gave_up(orc, emulate, c, g, h, n):
     assert rc == 0 and counts[2] == 1
     assert counts[1] == 0
     assert all(sorted(t[:-1]) == list(range(n)) and t[-1] == t[0] for t in tours)
+
+
+# A persistent launch initialises a barrier in the same place for ant after ant: each has to be
+# invalidated first.
+@pytest.mark.parametrize("c,g,h,n", [(36, 1, 32, 120), (12, 1, 32, 100), (36, 1, 8, 90),
+                                     (36, 2, 32, 200)])
+def test_barriers_end_with_their_ant(orc, emulate, c, g, h, n):
+    dist, choice = _instance(orc, n)
+    ants = 3 * (32 // h)
+    want = orc.construct(choice, dist, ants, seed=11, iteration=0)
+    rc, tours, _, counts = emulate(c, g, h, choice, dist, ants, [0, 0, 0], 11, n)
+    assert rc == 0 and np.array_equal(tours, want[0])
+    assert counts[2] == 0 and counts[3] == 0
