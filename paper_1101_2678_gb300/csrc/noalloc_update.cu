@@ -198,9 +198,10 @@ constexpr int kApplyTile = 32;
 
 __global__ void __launch_bounds__(256)
     noalloc_apply_kernel(float* tau, const float* __restrict__ heta, float* choice,
-                         const unsigned long long* __restrict__ acc,
-                         const unsigned long long* __restrict__ shift_slot, int n, float alpha,
-                         float rho) {
+                         const unsigned long long* acc, const unsigned long long* shift_slot,
+                         int n, float alpha, float rho) {
+  // (acc and shift_slot are still being written when this kernel starts: no
+  // __restrict__, whose read-only promise would hold for its whole life)
   __shared__ float dep[kApplyTile][kApplyTile + 1];
   const int bi = blockIdx.y, bj = blockIdx.x;
   const int tx = threadIdx.x, ty = threadIdx.y;
