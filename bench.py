@@ -472,13 +472,15 @@ def run_ours(args, w, rank, world, local):
         return
     peaks, peak_kind = measured_peaks()
     if args.variant == "acs":
-        kernel = "acs_rows_kernel"
+        kernel = "acs_construct_kernel" if args.nn else "acs_rows_kernel"
     elif args.nn:
         kernel = "construct_nn_kernel"
     elif args.selection != "eq1":
         kernel = "construct_rule_kernel"
-    elif n <= 240 and not (args.lanes_per_ant or args.warps_per_ant or args.ants_per_cta):
-        kernel = "construct_small_kernel"  # the whole matrix in shared memory
+    elif (n <= 232 or n <= 240 and m <= 608) and not (args.lanes_per_ant or args.warps_per_ant
+                                                       or args.ants_per_cta):
+        # the whole matrix in shared memory (small_warps in construct_small.cu)
+        kernel = "construct_small_kernel"
     else:
         kernel = "construct_phased_kernel"
     l2 = measure_l2_read_gbs()

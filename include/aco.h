@@ -83,7 +83,9 @@ extern "C" {
 #define ACO_OPT_PROFILE 4      /* 1: record CUDA events around every kernel     */
 #define ACO_OPT_WARPS_PER_ANT 5 /* 0 (default) = automatic, else 1, 2 or 4      */
 #define ACO_OPT_ANTS_PER_CTA 6 /* 0 (default) = automatic, else 1..32; at most 8
-                                  warps per CTA                                */
+                                  warps per CTA.  (Reads the walk's value also
+                                  where the small-instance construction, see
+                                  ACO_OPT_STAGING, runs.)                      */
 #define ACO_OPT_LANES_PER_ANT 7 /* 0 (default) = 32; 8 or 16: 32/H ants share a
                                   warp (one warp per ant group)                */
 #define ACO_OPT_SELECTION 8    /* ACO_SELECT_* below; default ACO_SELECT_EQ1     */
@@ -107,9 +109,10 @@ extern "C" {
                                   1 for n <= 64, else 0 (the faster measured
                                   on GB300).  Results are identical.  (With
                                   the default tiling, Eq. 1 instances of n <=
-                                  240 bring the whole choice_info matrix into
-                                  shared memory once per construction and
-                                  stage no rows.)                             */
+                                  240 - above 232 those with few ants, m <=
+                                  608 at n = 240 on 152 SMs - bring the whole
+                                  choice_info matrix into shared memory once
+                                  per construction and stage no rows.)        */
 
 #define ACO_SELECT_EQ1 0       /* Eq. 1 (random proportional rule), exact      */
 #define ACO_SELECT_DATA_PARALLEL 1 /* the paper's data-parallel kernel (Section

@@ -219,7 +219,7 @@ static int enqueue_construct(aco_colony* h) {
   if (!tiling_ok(t, h->I.rule)) return fail(ACO_EINVAL, "no construction tiling for n=%d", h->I.n);
   // the default tiling only: options that name a tiling get that one
   const bool small = h->I.rule == 0 && !h->warps_per_ant && !h->lanes_per_ant &&
-                     !h->ants_per_cta && construct_small_fits(h->I.n);
+                     !h->ants_per_cta && construct_small_fits(h->I.n, h->I.m, h->sms);
   cudaError_t e;
   if (h->profile && (e = record_event(h, h->ev[0], h->stream)) != cudaSuccess)
     return cuda_fail(e, "event");

@@ -1,21 +1,20 @@
 // Tour construction by Eq. 1 for instances whose whole choice_info matrix fits
-// in one CTA's shared memory (n <= 240).
+// in one CTA's shared memory (n <= 240, and few enough ants above n = 232).
 //
 // At these sizes a step is nothing but latency: the walk of
 // construct_phased.cuh spends a third of its step waiting for the row's copy
 // out of L2.  Here each CTA copies the matrix once (one bulk copy, a contiguous
 // n * ld floats) and a step starts with a 16-byte shared-memory load.  One warp
-// per ant, the ants spread over all SMs (as many per CTA as there are more
-// ants than SMs); lane l owns the cities [l*CH, l*CH + CH), CH = 4 up to
-// n = 128, else 8.  Every lane works out which of its cities would hold the
-// target; the votes that find the lane also carry the city's place in its
-// chunk, so a step has one warp scan, one shuffle and a few votes.  The search
-// is the single-precision one of eq1_phase() with its error bound, and
-// exact_pick() decides where that cannot.
+// per ant, the ants dealt evenly over all SMs; lane l owns the cities [l*CH,
+// l*CH + CH), CH = 4 up to n = 128, else 8.  Every lane works out which of its
+// cities would hold the target; the votes that find the lane also carry the
+// city's place in its chunk, so a step has one warp scan, one shuffle and a few
+// votes.  The search is the single-precision one of eq1_phase() with its error
+// bound, and exact_pick() decides where that cannot.
 // Construct, GB300, ms, m = n unless given, the walk -> this kernel: n = 24
 // 0.0176 -> 0.0118, n = 48 0.0286 -> 0.0172, n = 128 0.0708 -> 0.0373, n = 230
-// 0.134 -> 0.070, with m = 4864 0.253 -> 0.201: faster wherever it fits, so it
-// is taken there.  A step takes about 520 cycles, the scan and the votes most
+// 0.134 -> 0.070, with m = 4864 0.253 -> 0.201.  Which sizes take it is decided
+// by small_warps().  A step takes about 520 cycles, the scan and the votes most
 // of them.
 #include "construct.cuh"
 #include "kernels.h"
@@ -156,11 +155,30 @@ __global__ void __launch_bounds__(1024) construct_small_kernel(Instance I) {
 
 constexpr size_t kSmallMost = 227 * 1024;
 
+// Warps (ants) per CTA, one CTA on each SM at a time: the ants dealt evenly over
+// as few rounds of CTAs as the shared memory allows; 0 where the walk is taken.
+// From n = 233 on the matrix leaves room for fewer than 32 warps (233: 23,
+// 237: 8, 240: 2), and a round costs what its longest step does, so many ants
+// take many rounds.  Two rounds are still no slower than the walk, three are
+// not: ms, as many rounds as it takes / the walk / this rule, n = 240 with m =
+// 512 0.137 / 0.141 / 0.137, 1024 0.265 / 0.147 / 0.145, 4864 1.05 / 0.263 /
+// 0.259; n = 238, m = 1024 0.155 / 0.147 / 0.137.  Even rounds: n = 200, m =
+// 5000 (152 CTAs of 32 ants and 5 more) 0.337 / 0.245, of 17 ants 0.192.
+template <int CH>
+int small_warps(int n, int m, int sms) {
+  const int ld = (n + 3) / 4 * 4;
+  int most = 32;
+  while (most > 0 && small_bytes<CH>(n, ld, most) > kSmallMost) --most;
+  if (most == 0) return 0;
+  const int rounds = (m + sms * most - 1) / (sms * most);
+  if (most < 32 && rounds > 2) return 0;
+  return (m + sms * rounds - 1) / (sms * rounds);
+}
+
 template <int CH>
 cudaError_t launch_small(const Instance& I, int sms, cudaStream_t st) {
-  int warps = (I.m + sms - 1) / sms;
-  if (warps > 32) warps = 32;
-  while (warps > 1 && small_bytes<CH>(I.n, I.ld, warps) > kSmallMost) --warps;
+  const int warps = small_warps<CH>(I.n, I.m, sms);
+  if (warps < 1) return cudaErrorInvalidValue;
   static std::atomic<unsigned long long> done{0};
   const cudaError_t e = once_per_device(done, [] {
     return cudaFuncSetAttribute(construct_small_kernel<CH>,
@@ -174,9 +192,8 @@ cudaError_t launch_small(const Instance& I, int sms, cudaStream_t st) {
 
 }  // namespace
 
-bool construct_small_fits(int n) {
-  const int ld = (n + 3) / 4 * 4;
-  return n <= 256 && (n <= 128 ? small_bytes<4>(n, ld, 1) : small_bytes<8>(n, ld, 1)) <= kSmallMost;
+bool construct_small_fits(int n, int m, int sms) {
+  return n <= 256 && (n <= 128 ? small_warps<4>(n, m, sms) : small_warps<8>(n, m, sms)) > 0;
 }
 
 cudaError_t launch_construct_small(const Instance& I, int sms, cudaStream_t st) {

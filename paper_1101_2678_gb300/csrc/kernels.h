@@ -83,7 +83,7 @@ cudaError_t launch_construct_rule1(const Instance& I, ConstructTiling t, cudaStr
 cudaError_t launch_construct_rule2(const Instance& I, ConstructTiling t, cudaStream_t st);
 // Eq. 1 with the whole choice_info matrix in shared memory (construct_small.cu),
 // for the default tiling where construct_small_fits().
-bool construct_small_fits(int n);
+bool construct_small_fits(int n, int m, int sms);
 cudaError_t launch_construct_small(const Instance& I, int sms, cudaStream_t st);
 cudaError_t launch_construct_items(const Instance* insts, const int2* items, int count,
                                    ConstructTiling t, cudaStream_t st);
