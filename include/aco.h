@@ -534,12 +534,14 @@ int aco_pool_set_autotune(aco_pool_handle p, int32_t on);
  * each group of slots (a construction class, or all Ant Colony System
  * colonies), each group on its own stream with its own best and update
  * launches, where k = floor(T_max / T_group) within [1, 64] from a model of
- * one iteration's time alone (about n (0.6 + 0.025 n / 32) us; 4 n us for a
- * colony) and T_max that of the slowest group, and never more than the
- * iterations any slot of the group has left.  Short instances then keep
- * pace with the longest instead of waiting one long step per iteration.
- * Every slot still runs exactly its own iterations, so its results are
- * unchanged.  on = 0 (default): one iteration per step for every slot.
+ * one iteration's time alone (with k = n / 1000 about 5 + n (0.6 + 0.15 k^2)
+ * us, with lists 5 + n (0.52 + 0.03 k^2), for a colony 5 + n (1.15 + 0.21
+ * k^2), with lists 5 + n (1.15 + 0.18 k)) and T_max that of the slowest
+ * group, and never more than the iterations any slot of the group has left.
+ * Short instances then keep pace with the longest instead of waiting one
+ * long step per iteration.  Every slot still runs exactly its own
+ * iterations, so its results are unchanged.  on = 0 (default): one iteration
+ * per step for every slot.
  * ACO_EINVAL for a static batch (aco_batch_*), whose steps count iterations.
  * aco_pool_rate: the iterations the last step ran for `slot` (live or
  * finished; 1 unless multi-rate; ACO_ESTATE before its first step).

@@ -230,11 +230,18 @@ static int ensure_capacity(void** ptr, size_t* cap, size_t need, size_t elem) {
 }
 
 // Modelled time of one iteration of an instance of n cities run alone, in
-// microseconds: n dependent steps, each costing a fixed latency plus the
-// per-lane chunk (n / 32 cities); the Ant Colony System's lockstep step is
-// about 4 us.  Only ratios matter (they set the iterations per step).
-static double iteration_time_model(int n, bool acs, bool nn = false) {
-  return acs ? 4.0 * n : nn ? 0.65 * n : n * (0.6 + 0.025 * n / 32.0);
+// microseconds: the launches, and n dependent steps, each a fixed latency and a
+// part that grows with the row.  Only ratios matter (they set the iterations
+// per step).  GB300, one slot in a pool, m = n or 10 ants, us measured / model:
+//   Eq. 1       n = 100 65 / 65, 300 185 / 189, 1002 816 / 757, 2392 3430 / 3490
+//   with lists  n = 100 63 / 57, 300 157 / 162, 1002 562 / 556, 2392 1690 / 1660
+//   colonies    n = 100 113 / 120, 300 363 / 356, 1002 1430 / 1370, 2392 5730 / 5630
+//   with lists  n = 100 115 / 122, 300 376 / 366, 1002 1400 / 1340, 2392 3680 / 3790
+static double iteration_time_model(int n, bool acs, bool nn) {
+  const double k = n / 1000.0;
+  const double step = acs ? (nn ? 1.15 + 0.18 * k : 1.15 + 0.21 * k * k)
+                          : (nn ? 0.52 + 0.03 * k * k : 0.6 + 0.15 * k * k);
+  return 5.0 + n * step;
 }
 constexpr int kMaxRate = 64;  // iterations per step at most
 
@@ -274,6 +281,7 @@ static int pool_rebuild(aco_pool* p) {
   // Ant Colony System slots: one CTA per colony in one launch of their own
   // (MAX-MIN Ant System slots construct and update with the Ant System ones:
   // the best and row-update kernels follow each slot's rule)
+  int acs_n[2] = {0, 0};  // largest colony without and with lists
   for (int pass = 0; pass < 2; ++pass) {
     for (int s : live) {
       const PoolSlot& sl = p->slots[(size_t)s];
@@ -281,6 +289,7 @@ static int pool_rebuild(aco_pool* p) {
       p->h_acs.push_back(s);
       p->acs_max_m = std::max(p->acs_max_m, sl.m);
       p->acs_max_n = std::max(p->acs_max_n, sl.n);
+      acs_n[pass] = std::max(acs_n[pass], sl.n);
     }
     if (pass == 0) p->acs_dense = (int)p->h_acs.size();
   }
@@ -335,7 +344,11 @@ static int pool_rebuild(aco_pool* p) {
     p->classes.push_back(c);
   }
   // iterations per step of each group (1 unless multi-rate stepping is on)
-  double t_max = p->h_acs.empty() ? 0.0 : iteration_time_model(p->acs_max_n, true);
+  // (the colonies without lists and those with them follow each other)
+  double t_acs = 0.0;
+  for (int pass = 0; pass < 2; ++pass)
+    if (acs_n[pass]) t_acs += iteration_time_model(acs_n[pass], true, pass == 1);
+  double t_max = t_acs;
   for (const auto& c : p->classes)
     t_max = std::max(t_max, iteration_time_model(c.max_n, false, c.nn));
   for (auto& c : p->classes) {
@@ -345,8 +358,7 @@ static int pool_rebuild(aco_pool* p) {
       p->slots[(size_t)p->h_cls_slots[(size_t)(c.slot_begin + i)]].rate = c.k;
   }
   p->acs_k = p->h_acs.empty() ? 1
-                              : group_rate(p, p->h_acs.data(), (int)p->h_acs.size(),
-                                           iteration_time_model(p->acs_max_n, true), t_max);
+                              : group_rate(p, p->h_acs.data(), (int)p->h_acs.size(), t_acs, t_max);
   for (int s : p->h_acs) p->slots[(size_t)s].rate = p->acs_k;
   int rc = ensure_capacity((void**)&p->d_items, &p->items_cap, p->h_items.size(), sizeof(int2));
   if (!rc) rc = ensure_capacity((void**)&p->d_rows, &p->rows_cap, p->h_rows.size(), sizeof(int2));
