@@ -593,8 +593,9 @@ int aco_batch_destroy(aco_batch b);
  * that reserve all device memory up front.  It performs the same update as
  * aco_update_pheromone with ACO_DEPOSIT_ATOMIC_U64 (same results bit for
  * bit), but on arrays the caller owns and with its scratch (a 64-bit
- * accumulator of ACO_NOALLOC_MAX_N^2 entries, about 8.4 MB) in one static device array that the library
- * reserves on every GPU that loads it, until the process exits.
+ * accumulator of ACO_NOALLOC_MAX_N^2 entries, about 8.4 MB) in one static
+ * device array that the library reserves on every GPU that loads it, until
+ * the process exits.
  * ======================================================================== */
 #define ACO_NOALLOC_MAX_N 1024
 #define ACO_NOALLOC_MAX_M 4096

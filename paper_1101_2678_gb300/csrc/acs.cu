@@ -331,7 +331,7 @@ __device__ __forceinline__ void fence_proxy_async_global() {
 // 0.374 / 0.200 / 0.221, n = 517 1.29 / 1.01 / 0.66, n = 1002 3.89 / 2.32 /
 // 1.42, n = 2392 14.3 / 11.3 / 5.69, n = 4096 35.8 / 35.3 / 18.1 (loads by ten
 // warps queue in the SM's load unit for 1400 cycles of a step at n = 1002); a
-// step of 256 colonies 4.59 / 2.89 / 1.82.
+// step of 256 colonies 4.59 / 2.89 / 1.84.
 template <int B>
 __device__ __forceinline__ void acs_rows_body(const Instance& I, uint32_t* acs_seen,
                                               uint32_t* s_edge, float* s_choice,
@@ -689,6 +689,11 @@ static bool launch_acs_rows(ChunkList<Bs...>, const Instance& I, cudaStream_t st
           ...);
 }
 
+// One block width for all colonies of the launch, that of the largest.  A step,
+// ms, every pass over the rows from L1 -> this: 256 colonies of n = 100 0.65 ->
+// 0.57, one of 1002 and 600 of 100 5.10 -> 2.48, one of 2392 and 1000 of 100
+// 17.0 -> 7.6, one of 4096 and 800 of 200 39.7 -> 20.5, four of 600 and 1000 of
+// 200 3.65 -> 3.65 (nowhere slower).
 template <int... Bs>
 static bool launch_acs_rows_slots(ChunkList<Bs...>, const Instance* insts, const int* slots,
                                   int count, int max_m, int max_n, cudaStream_t st) {

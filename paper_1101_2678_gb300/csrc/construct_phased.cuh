@@ -28,8 +28,8 @@
 //
 // Construct, GB300, ms, m = n unless given: quantised 64-bit sums -> this
 // walk: n = 48 0.034 -> 0.029, n = 200 0.163 -> 0.116, n = 384 0.310 -> 0.222,
-// n = 517 0.464 -> 0.317, n = 1002 1.118 -> 0.782, n = 1500 2.13 -> 1.40,
-// n = 2392 5.05 -> 3.24, n = 4096 with m = 1024 9.02 -> 6.16.  Small instances
+// n = 517 0.464 -> 0.313, n = 1002 1.118 -> 0.762, n = 1500 2.13 -> 1.37,
+// n = 2392 5.05 -> 3.20, n = 4096 with m = 1024 9.02 -> 6.12.  Small instances
 // are bound by the step's chain (about 1500 cycles at n = 1002: the row copy
 // 500, the sums 200, the scan and the lane 280, the slot 150, the rest
 // issue), large ones also by the rows: 54.7 GB at n = 2392 take 2.7 ms at the
@@ -111,8 +111,8 @@ __device__ __forceinline__ Pick exact_pick(const float* row, uint16_t* list, int
     // Every open weight is zero: the lowest open city (a list's smallest
     // entry; zero_entry is above every city's).
     uint32_t cand = 0xffffffffu;
-  #pragma unroll 1
-  for (int i = cp - 1; i >= 0; --i) {
+#pragma unroll 1
+    for (int i = cp - 1; i >= 0; --i) {
       if (list) {
         cand = min(cand, (uint32_t)list[tg * cp + i]);
       } else {
